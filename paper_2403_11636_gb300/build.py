@@ -21,7 +21,7 @@ LIB = os.path.join(HERE, "libfc.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["fc_geom.cu", "fc_assemble.cu", "fc_mg.cu", "fc_patch.cu", "fc_api.cu", "fc_noalloc.cu", "fc_batch.cu",
-           "fc_probe.cu", "fc_q2.cu", "fc_amr.cu"]
+           "fc_probe.cu", "fc_q2.cu", "fc_amr.cu", "fc_digits.cu"]
 EXTRA = {"fc_geom.cu": ["--fmad=false"], "fc_amr.cu": ["-Xcompiler", "-ffp-contract=off"]}
 
 
@@ -41,7 +41,7 @@ def _stale(target: str, deps) -> bool:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, "fc_internal.cuh"), os.path.join(INCLUDE, "fc.h")]
+    headers = [os.path.join(CSRC, "fc_internal.cuh"), os.path.join(CSRC, "fc_node.cuh"), os.path.join(INCLUDE, "fc.h")]
     nvcc = _nvcc()
 
     def compile_one(src):

@@ -295,7 +295,7 @@ fc_status smoother_residual(fc_handle h, int li, const double* x, const double* 
   } else if (h->opt.cache == FC_CACHE_INVERSE && (h->opt.prec == FC_PREC_FP32 || h->opt.prec == FC_PREC_BF16)) {
     CK(launch_residual_f32(L.g, L.st, L.mask, x, b, L.rpad32, h->stream));
   } else {
-    CK(launch_residual(L.g, L.st, L.mask, x, b, nullptr, L.rpad, h->stream));
+    CK(residual_fp64(L, x, b, nullptr, L.rpad, h->stream));
   }
   return FC_OK;
 }
@@ -370,8 +370,7 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
     if (h->opt.cache == FC_CACHE_INVERSE) {
       ProfScope ps(h, 0, level_apply_bytes(h, li));
       ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, level_apply_bytes(h, li));
-      CK(launch_patch_apply(L.g, h->opt.prec, L.coef, L.mask, L.rpad, L.rpad32, h->opt.omega, x, L.prow,
-                            h->stream));
+      CK(apply_rows(L, h->opt.prec, L.rpad, L.rpad32, h->opt.omega, x, h->stream));
     } else if (h->opt.cache == FC_CACHE_MATRIX) {
       ProfScope ps(h, 0, (double)L.fac_bytes);
       CK(launch_factor_apply(L.g, L.st, factor_store(L), L.mask, L.rpad, h->opt.omega, x, L.prow, h->stream));
@@ -385,6 +384,53 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
 }
 
 fc_status vcycle_level(fc_handle h, int li, double* x, const double* b);
+
+// Class products of a level on the tensor cores (fc_digits.cu): the plan is
+// kept where it pays.
+bool digit_level(const LevelGeom& G, int kind) {
+  if (G.dim == 3) return kind == 0 && G.nnodes >= kDigitApply3;
+  return G.nnodes >= (kind == 0 ? kDigitApply2 : kDigitResidual2);
+}
+
+void free_digit_plan(fc_handle h, DigitPlan* p) {
+  dfree(h, p->cls);
+  dfree(h, p->list);
+  dfree(h, p->rows);
+  dfree(h, p->w);
+  dfree(h, p->sc);
+  *p = DigitPlan();
+}
+
+fc_status make_digit_plan(fc_handle h, Level& L, int kind, const double* src, const unsigned char* nclass) {
+  const LevelGeom& G = L.g;
+  DigitPlan& p = L.dig[kind];
+  const int part = kind == 0 ? 1 : 0;
+  const size_t before = h->bytes[part];
+  unsigned char* tmp = nullptr;
+  int *rep = nullptr, *counts = nullptr;
+  char *rows = nullptr, *w = nullptr;
+  CK(dalloc(h, &p.cls, (size_t)G.nnodes, part));
+  CK(dalloc(h, &p.list, (size_t)G.nnodes, part));
+  CK(dalloc(h, &rows, digit_plan_rows_bytes(G.dim, kind), part));
+  p.rows = (uint4*)rows;
+  CK(dalloc(h, &w, digit_plan_w_bytes(G.dim, kind), part));
+  p.w = (double*)w;
+  CK(dalloc(h, &p.sc, 2, part));
+  CK(dalloc(h, &tmp, (size_t)G.nnodes, -1));
+  CK(dalloc(h, &rep, 6, -1));
+  CK(dalloc(h, &counts, (size_t)digit_plan_counts(G.nnodes), -1));
+  p.err = h->d_err;
+  CK(build_digit_plan(G, kind, src, nclass, L.mask, L.prow, &p, tmp, rep, counts, h->stream));
+  dfree(h, tmp);
+  dfree(h, rep);
+  dfree(h, counts);
+  p.on = G.nnodes - p.nlist >= G.nnodes / 16;
+  if (!p.on) {
+    free_digit_plan(h, &p);
+    h->bytes[part] = before;
+  }
+  return FC_OK;
+}
 
 // Restriction of the finest residual buffer and the whole coarser V-cycle,
 // all on buffers fixed per handle: captured once into a CUDA graph (one
@@ -504,7 +550,7 @@ cudaError_t level_residual(fc_handle h, int li, const double* x, const double* b
   if (amr_path(h)) return launch_amr_residual(L.amr, x, b, r, h->stream);
   if (q2_path(h))
     return launch_q2_residual(h->dim, L.q2, L.q2A, L.q2B, L.q2T, L.q2mask, x, b, r, nullptr, nullptr, h->stream);
-  return launch_residual(L.g, L.st, L.mask, x, b, r, nullptr, h->stream);
+  return residual_fp64(L, x, b, r, nullptr, h->stream);
 }
 
 cudaError_t level_restrict(fc_handle h, int li, const double* rf, double* bc) {
@@ -865,6 +911,9 @@ size_t fc_footprint_estimate(const fc_grid* g, int depth, const fc_options* o) {
       cells *= n;
     }
     const size_t dof = nodes * nd, pv = pad * nd;
+    // class products: node classes, list of the other nodes, rows (two plans)
+    for (int kind = 0; kind < (dim == 2 ? 2 : 1); ++kind)
+      held += nodes * 5 + 128 + digit_plan_rows_bytes(dim, kind) + digit_plan_w_bytes(dim, kind);
     if (l == 0) coarse_dof = dof;
     if (l == depth - 1) fine_dof = dof;
     held += nodes * nb * sp * 8 + nodes + dof * 8;                  // stencil, mask, Dirichlet values
@@ -1060,6 +1109,20 @@ fc_status fc_setup(fc_handle* out, const fc_grid* g, const fc_levelset* ls, doub
       CK(launch_dead_layers(G, L.mask, L.dead, h->stream));
       L.g.dead_layer = L.dead;
     }
+    // ---- class products: the FP64 operator of the levels that use it (the
+    // reduced-precision V-cycles only on the finest level, for FGMRES)
+    unsigned char* dig_nclass = nullptr;
+    const bool dig_fp64 = o->cache != FC_CACHE_INVERSE || o->prec == FC_PREC_FP64;
+    const bool dig_res = digit_level(G, 1) && (dig_fp64 || li == depth - 1);
+    const bool dig_apply = digit_level(G, 0) && li > 0 && o->cache == FC_CACHE_INVERSE && o->prec == FC_PREC_FP64;
+    if (dig_res || dig_apply) {
+      CK(dalloc(h, &dig_nclass, (size_t)G.nnodes, -1));
+      CK(launch_node_classes(G, cclass, dig_nclass, h->stream));
+      if (dig_res) {
+        const fc_status ds = make_digit_plan(h, L, 1, L.st, dig_nclass);
+        if (ds != FC_OK) return ds;
+      }
+    }
     // ---- vectors
     long long padn = pad_nodes(G);
     CK(dalloc(h, &L.x, (size_t)G.ndof, 2));
@@ -1248,6 +1311,10 @@ fc_status fc_setup(fc_handle* out, const fc_grid* g, const fc_levelset* ls, doub
         if (o->prec == FC_PREC_FP64) {
           L.coef = c64;
           L.coef_bytes = n * 8;
+          if (dig_apply) {
+            const fc_status ds = make_digit_plan(h, L, 0, c64, dig_nclass);
+            if (ds != FC_OK) return ds;
+          }
         } else {
           size_t eb = coef_elem_bytes(o->prec);
           void* cv = nullptr;
@@ -1329,6 +1396,7 @@ fc_status fc_setup(fc_handle* out, const fc_grid* g, const fc_levelset* ls, doub
       st = check_err(h);
       if (st != FC_OK) return st;
     }
+    dfree(h, dig_nclass);
     if (galerkin) {
       dfree(h, fine_estat);
       fine_estat = estat;
@@ -1720,6 +1788,7 @@ fc_status fc_destroy(fc_handle h) {
     dfree(h, L.x); dfree(h, L.b); dfree(h, L.r); dfree(h, L.rpad); dfree(h, L.rpad32);
     dfree(h, L.st2); dfree(h, L.xp2); dfree(h, L.bp2); dfree(h, L.prow);
     dfree(h, L.st32); dfree(h, L.d32); dfree(h, L.b32);
+    free_digit_plan(h, &L.dig[0]); free_digit_plan(h, &L.dig[1]);
     dfree(h, L.q2mask); dfree(h, L.q2A); dfree(h, L.q2B); dfree(h, L.q2T); dfree(h, L.q2rpv); dfree(h, L.q2rpp);
     dfree(h, L.amr.rowptr); dfree(h, L.amr.col); dfree(h, L.amr.val); dfree(h, L.amr.fixed);
     dfree(h, L.amr.pstart); dfree(h, L.amr.pdof); dfree(h, L.amr.pown);

@@ -463,6 +463,15 @@ cudaError_t launch_patch_classes(const LevelGeom& g, const unsigned char* cclass
 }
 
 
+cudaError_t launch_node_classes(const LevelGeom& g, const unsigned char* cclass, unsigned char* nclass,
+                                cudaStream_t s) {
+  const unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
+  if (g.dim == 2) node_class_kernel<2><<<blocks, 256, 0, s>>>(g, cclass, nclass);
+  else node_class_kernel<3><<<blocks, 256, 0, s>>>(g, cclass, nclass);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_galerkin(const LevelGeom& gc, const LevelGeom& gf, const double* stf, const unsigned char* maskf,
                             double* stc, cudaStream_t s) {
   const long long n = gc.nnodes * (gc.dim == 3 ? 27 : 9);

@@ -1,0 +1,952 @@
+// fc_digits.cu -- FP64 products with rows that many nodes share, on the tensor
+// cores.
+//
+// Away from obstacles and walls the operator's stencil and the cached patch
+// rows are the same for every node of a class (fluid or fictitious), so the
+// smoother residual y = L x and the patch apply y = Inv r are products of one
+// short matrix W (d+1 rows; 27 or 59 slots in 2D, 402 for the patch in 3D) with
+// vectors gathered around each node.  FP64 is the bound of both on this part
+// (a warp FMA takes 64 clocks of an SM partition), so the products are formed
+// exactly from digits:
+//
+//  - a CTA takes a tile of nodes and its halo, finds the largest exponent E of
+//    the values that the tile's products read, and writes each value as a
+//    62-bit fixed-point number v 2^(62-E) in eight signed base-256 digits,
+//    held as half-precision integers in [-128, 127];
+//  - the rows W have the same form with an exponent per row (setup), the
+//    velocity and pressure columns first brought to one scale by a power of
+//    two (delta), as D L D equilibrates the blocks;
+//  - S_d = sum_slots sum_{s+t=d} w_s v_t, d = 0..7, is one matrix product: a
+//    node is a row of the left operand (K = slot, digit), a row of W and an
+//    antidiagonal d a column of the right one (w_{d-s} at digit s), and
+//    y = 2^(Ew+E-12) sum_d S_d 2^(-8d), rounded to double once.
+//
+// The digits of a component lie 16 bytes a node, nodes in the order of the
+// halo tile, so the left operand of a pair of slots is read in place: 128
+// consecutive nodes are a tcgen05 tile, a slot is an offset of its descriptor
+// (8 x 16-byte core matrices 128 bytes apart; the second slot at the leading
+// offset).  Rows of the halo are computed too and dropped.  Accumulators stay
+// in tensor memory; a thread then reads all S_d of one node.
+//
+// Exactness: products are integers of at most 2^14 and float32 sums of
+// integers are exact below 2^24.  digit_rows_kernel adds up the magnitudes of
+// W's digits: the sums d <= 5 cannot reach 2^24 (or the class is not used);
+// those of d = 6, 7, of weight 2^-48 and less, could round by a unit.  With
+// the antidiagonals that are left out (2^-64) the result is the dot product of
+// the stored doubles to 2^-51 of max|w| max|v|, in practice to 2^-60, where a
+// chain of FP64 fused multiply-adds rounds each partial sum to 2^-53.  A tile
+// that holds an infinity or NaN, or whose exponent is extreme, takes plain
+// FP64 products (fp64_product).
+//
+// Which nodes: `cls` of the plan.  A node read by products of both classes
+// would need two scales; the products that read one are left, with all other
+// nodes, to the FP64 kernels (plan list).
+#include <cuda_fp16.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "fc_node.cuh"
+
+namespace fc {
+
+namespace {
+
+// KIND 0: patch apply (velocities of the 5^d box, pressures of the 3^d box),
+// KIND 1: operator (all components of the 3^d box; 2D: in 3D the tile's halo
+// and the rows of the halo cost more than the 270 FMA of a node).
+template <int DIM, int KIND>
+struct Dig {
+  static constexpr int ND = DIM + 1, R = KIND == 0 ? 2 : 1;
+  static constexpr int NSLOT = KIND == 0 ? SlotDims<DIM>::NSLOT : (DIM == 3 ? 27 : 9) * ND;
+  static constexpr int STEPS = (NSLOT + 1) / 2;  // K = 16: two slots
+  // tile: NBLK blocks of 128 rows cover the tile's nodes in halo order
+  static constexpr int TX = DIM == 3 ? 16 : 32, TY = DIM == 3 ? 8 : 14, TZ = DIM == 3 ? 4 : 1;
+  static constexpr int HX = TX + 2 * R, HY = TY + 2 * R, HZ = DIM == 3 ? TZ + 2 * R : 1;
+  static constexpr int NHALO = HX * HY * HZ;
+  static constexpr int LAST = (TX - 1) + HX * ((TY - 1) + HY * (TZ - 1));
+  static constexpr int NBLK = LAST / 128 + 1;
+  static constexpr int TMEM = NBLK * 32 <= 128 ? 128 : NBLK * 32 <= 256 ? 256 : 512;  // columns
+  // largest offset of a slot's node from the corner, and the nodes of a plane
+  // that some row of a block can read
+  static constexpr int FAR = 2 * R * (1 + HX + (DIM == 3 ? HX * HY : 0));
+  static constexpr int PLANE = NBLK * 128 + FAR + 8;
+  static constexpr int THREADS = 256;
+  static constexpr int N = 32;  // columns: 4 rows x 8 antidiagonals (2D: the fourth row is zero)
+  // W is read in pieces of CS steps, NST pieces in flight (1 KB a step)
+  static constexpr int CS = DIM == 3 ? 18 : STEPS, NST = DIM == 3 ? 3 : 1, NCH = (STEPS + CS - 1) / CS;
+  static constexpr size_t O_ROWS = (size_t)PLANE * 16 * ND;
+  static constexpr size_t O_OFFS = O_ROWS + (size_t)NST * CS * 1024;
+  static constexpr size_t O_CLS = O_OFFS + (size_t)STEPS * sizeof(unsigned);
+  static constexpr size_t BYTES = (O_CLS + NHALO + 15) / 16 * 16;
+};
+
+// Slots in the order of their digits' addresses (component, then node).
+// Offset of the slot's node, its component; the slot's index in the cached
+// rows (KIND 0) or in (node, component) order (KIND 1)
+template <int DIM, int KIND>
+__device__ __forceinline__ void slot_of(int j, int* o, int* c, int* src) {
+  using P = SlotDims<DIM>;
+  constexpr int NV = KIND == 0 ? P::NU : (DIM == 3 ? 27 : 9);
+  int t, w, h;
+  if (j < NV * DIM) {
+    *c = j / NV;
+    t = j % NV;
+    w = KIND == 0 ? 5 : 3;
+  } else {
+    *c = DIM;
+    t = j - NV * DIM;
+    w = 3;
+  }
+  h = w / 2;
+  o[0] = t % w - h;
+  o[1] = DIM == 3 ? (t / w) % w - h : t / w - h;
+  o[2] = DIM == 3 ? t / (w * w) - h : 0;
+  if (KIND == 0) *src = *c < DIM ? t * DIM + *c : P::NU * DIM + t;
+  else *src = t * (DIM + 1) + *c;
+}
+
+// eight base-256 digits of V + 0x80..80 (most significant first), as halves
+__device__ __forceinline__ uint4 digits_of(long long V) {
+  const unsigned long long T = (unsigned long long)V + 0x8080808080808080ull;
+  const unsigned hi = (unsigned)(T >> 32), lo = (unsigned)T;
+  // 0x6400 + u is the half 1024 + u; less 1152 leaves the digit u - 128
+  const __half2 m = __half2half2(__ushort_as_half(0x6480));
+  unsigned w[4] = {__byte_perm(hi, 0x64646464u, 0x4243), __byte_perm(hi, 0x64646464u, 0x4041),
+                   __byte_perm(lo, 0x64646464u, 0x4243), __byte_perm(lo, 0x64646464u, 0x4041)};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    __half2 h = *reinterpret_cast<__half2*>(&w[k]);
+    h = __hsub2(h, m);
+    w[k] = *reinterpret_cast<unsigned*>(&h);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// v 2^(62 - E) truncated, for |v| < 2^E with E = emax - 1022 and e the biased
+// exponent of v (shifted by delta for pressures)
+__device__ __forceinline__ long long fixed_point(double v, int emax, int shift) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  if (e == 0) return 0;  // zero or subnormal
+  const int sh = emax - (e + shift);
+  if (sh > 62) return 0;
+  const unsigned long long m = ((((unsigned long long)(hi & 0xfffffu) | 0x100000ull) << 32) | lo) << 9;
+  const long long V = (long long)(m >> sh);
+  return (hi >> 31) ? -V : V;
+}
+
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// ---- tcgen05, mbarrier and bulk copies
+constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait that takes a second gives up
+
+__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+  unsigned long long start = 0ull;
+  for (;;) {
+    unsigned done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    unsigned long long now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (start == 0ull) start = now;
+    else if (now - start > kWaitNs) return false;
+  }
+}
+// global -> shared copy of `bytes` (a multiple of 16) that completes on bar
+__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void tc_mma(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc,
+                                       bool add) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"((unsigned)add)
+      : "memory");
+}
+// one lane of a full warp; a branch on it keeps the descriptors in uniform
+// registers (43 clocks from product to product; 84 behind a test of threadIdx)
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0u;
+}
+__device__ __forceinline__ void tc_commit(unsigned bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_load32(unsigned addr, unsigned* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(addr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+struct DigArgs {
+  const unsigned char* cls;
+  const uint4* rows;
+  const double* w;
+  const DigitScale* sc;
+  unsigned* err;
+  const int* list;
+  int nlist, list_blocks;
+  // KIND 0: v = padded residual, x updated.  KIND 1: v = x, r and rpad
+  // (nullable) receive b - L x (L x when b is null)
+  const double* v;
+  const double* b;
+  double* x;
+  double* r;
+  double* rpad;
+  double omega;
+  // the FP64 products of the list
+  const double* coef;  // KIND 0 rows, KIND 1 stencil
+  const unsigned char* mask;
+  const int* prow;
+};
+
+// y of node i in plain FP64 (W by class)
+template <int DIM, int KIND>
+__device__ void fp64_product(const LevelGeom& g, const double* __restrict__ w, const double* __restrict__ v,
+                             const int* ia, double* y) {
+  using D = Dig<DIM, KIND>;
+  for (int c = 0; c < D::ND; ++c) y[c] = 0.0;
+  for (int j = 0; j < D::NSLOT; ++j) {
+    int o[3], c, src;
+    slot_of<DIM, KIND>(j, o, &c, &src);
+    const int i0 = ia[0] + o[0], i1 = ia[1] + o[1], i2 = ia[2] + o[2];
+    const long long n = KIND == 0 ? pad_node(g, i0, i1, i2)
+                                  : i0 + (long long)g.nn[0] * (i1 + (long long)(DIM == 3 ? g.nn[1] : 1) * i2);
+    const double t = v[n * D::ND + c];
+    for (int q = 0; q < D::ND; ++q) y[q] = y[q] + w[(size_t)j * D::ND + q] * t;
+  }
+}
+
+// x + omega y (own = x, scale includes omega), or b - y (own = b; y without b)
+template <int DIM, int KIND>
+__device__ __forceinline__ void store_product(const LevelGeom& g, const DigArgs& a, const int* ia, const double* own,
+                                              const double* y, const double* scale) {
+  constexpr int ND = DIM + 1;
+  const long long n = ia[0] + (long long)g.nn[0] * (ia[1] + (long long)(DIM == 3 ? g.nn[1] : 1) * ia[2]);
+  double v[ND];
+#pragma unroll
+  for (int c = 0; c < ND; ++c) {
+    if (KIND == 0) v[c] = own[c] + scale[c] * y[c];
+    else v[c] = a.b ? own[c] - scale[c] * y[c] : scale[c] * y[c];
+  }
+  if (KIND == 0) {
+#pragma unroll
+    for (int c = 0; c < ND; ++c) a.x[n * ND + c] = v[c];
+    return;
+  }
+  if (a.r) {
+#pragma unroll
+    for (int c = 0; c < ND; ++c) a.r[n * ND + c] = v[c];
+  }
+  if (a.rpad) {
+    double* p = a.rpad + pad_node(g, ia[0], ia[1], ia[2]) * ND;
+#pragma unroll
+    for (int c = 0; c < ND; ++c) p[c] = v[c];
+  }
+}
+
+// 2D: the first list_blocks CTAs take the nodes of the plan's list in FP64.
+// The others take a tile each.  (CTAs that keep W and walk over the tiles, the
+// next tile's values loaded during the products, were slower: 196 against 164
+// us for the 1537^2 patch apply.)
+template <int DIM, int KIND>
+__global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
+    digit_product_kernel(LevelGeom g, DigArgs a, int tiles_x, int tiles_y) {
+  using D = Dig<DIM, KIND>;
+  constexpr int ND = D::ND, R = D::R;
+  extern __shared__ uint4 dsm[];
+  if (DIM == 2 && (int)blockIdx.x < a.list_blocks) {
+    if constexpr (KIND == 0) {
+      constexpr int TPP = 4;
+      int* soff = reinterpret_cast<int*>(dsm);
+      slot_table<DIM>(g, soff);
+      const int gi = (int)((blockIdx.x * 256u + threadIdx.x) / TPP);
+      const bool valid = gi < a.nlist;
+      apply_fp64_patch<DIM, TPP>(g, a.coef, a.mask, a.v, a.omega, a.x, a.prow, soff,
+                                 (unsigned)a.list[valid ? gi : a.nlist - 1], valid);
+    } else {
+      constexpr int TPP = 4;
+      const int t = (int)((blockIdx.x * 256u + threadIdx.x) / TPP);
+      const bool valid = t < a.nlist;
+      residual_node<DIM, 0, TPP>(g, a.coef, a.mask, a.v, a.b, a.r, a.rpad, nullptr, a.list[valid ? t : a.nlist - 1],
+                                 valid);
+    }
+    return;
+  }
+  char* smem = reinterpret_cast<char*>(dsm);
+  unsigned* soffs = reinterpret_cast<unsigned*>(smem + D::O_OFFS);
+  unsigned char* scls = reinterpret_cast<unsigned char*>(smem + D::O_CLS);
+  constexpr int NH = (D::NHALO + D::THREADS - 1) / D::THREADS;
+  // W arrived [NST], W used [NST], products done [per block where W is one piece]
+  constexpr int NDONE = D::NCH == 1 ? D::NBLK : 1;
+  __shared__ __align__(8) unsigned long long sbar[2 * D::NST + NDONE];
+  __shared__ int semax[2], sbad, sfail;
+  __shared__ unsigned sblk[2], stmem;
+  const int tid = threadIdx.x, lane = tid & 31, wib = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem);
+  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(sbar);
+  const unsigned bar_done = bar0 + 8 * 2 * D::NST;
+  const unsigned tile = blockIdx.x - (unsigned)a.list_blocks, tq = tile / (unsigned)tiles_x;
+  // the first R layers of a grid hold no class node (their boxes leave it): of
+  // 2^k + 1 nodes, a multiple of the tile and a remainder are left
+  const int bx = (int)(tile - tq * (unsigned)tiles_x) * D::TX + R;
+  const int by = (int)(DIM == 3 ? tq % (unsigned)tiles_y : tq) * D::TY + R;
+  const int bz = DIM == 3 ? (int)(tq / (unsigned)tiles_y) * D::TZ + R : 0;
+  // ---- the tile and its halo: every load is issued before the first is used
+  unsigned char hc[NH];
+  double hv[NH][ND];
+#pragma unroll
+  for (int q = 0; q < NH; ++q) {
+    const int n = q * D::THREADS + tid;
+    const int hx = n % D::HX, hy = (n / D::HX) % D::HY, hz = n / (D::HX * D::HY);
+    const int i = bx + hx - R, j = by + hy - R, k = DIM == 3 ? bz + hz - R : 0;
+    const bool in =
+        n < D::NHALO && i >= 0 && i < g.nn[0] && j >= 0 && j < g.nn[1] && (DIM == 2 || (k >= 0 && k < g.nn[2]));
+    const long long at = in ? i + (long long)g.nn[0] * (j + (long long)(DIM == 3 ? g.nn[1] : 1) * k) : 0;
+    const double* v = a.v + (KIND == 0 ? (in ? pad_node(g, i, j, k) : 0) : at) * ND;
+    hc[q] = in ? a.cls[at] : (unsigned char)0;
+    if (KIND == 0 && ND == 4) {  // (own buffer: 16-byte aligned; x is the caller's)
+      const double2 v0 = in ? reinterpret_cast<const double2*>(v)[0] : make_double2(0.0, 0.0);
+      const double2 v1 = in ? reinterpret_cast<const double2*>(v)[1] : make_double2(0.0, 0.0);
+      hv[q][0] = v0.x; hv[q][1] = v0.y; hv[q][2] = v1.x; hv[q][ND - 1] = v1.y;
+    } else {
+#pragma unroll
+      for (int c = 0; c < ND; ++c) hv[q][c] = in ? v[c] : 0.0;
+    }
+  }
+  const int delta[2] = {a.sc[0].delta, a.sc[1].delta};
+  const bool sc_ok[2] = {a.sc[0].ok != 0, a.sc[1].ok != 0};
+  if (tid == 0) {
+    for (int k = 0; k < 2 * D::NST + NDONE; ++k) mbar_init(bar0 + 8 * k, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    semax[0] = semax[1] = -100000;
+    sblk[0] = sblk[1] = 0u;
+    sbad = 0;
+    sfail = 0;
+  }
+  // operand offsets of a step: first slot's digits, and the second's distance
+  for (int t = tid; t < D::STEPS; t += D::THREADS) {
+    unsigned at[2];
+    for (int h = 0; h < 2; ++h) {
+      int o[3], c, src;
+      const int j = 2 * t + h;
+      slot_of<DIM, KIND>(j < D::NSLOT ? j : j - 1, o, &c, &src);
+      at[h] = (unsigned)(c * D::PLANE + (o[0] + R) + D::HX * ((o[1] + R) + (DIM == 3 ? D::HY * (o[2] + R) : 0)));
+      if (j >= D::NSLOT) at[h] += 1;  // an odd count's last slot: any digits, W's are zero
+    }
+    soffs[t] = at[0] | ((at[1] - at[0]) << 16);  // in units of 16 bytes
+  }
+  // past the halo: zeros, read by rows whose results are dropped
+  for (int t = tid; t < (D::PLANE - D::NHALO) * ND; t += D::THREADS) {
+    const int c = t / (D::PLANE - D::NHALO), n = D::NHALO + t % (D::PLANE - D::NHALO);
+    *reinterpret_cast<uint4*>(smem + ((size_t)c * D::PLANE + n) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  // W in pieces of CS steps through NST places
+  auto load_w = [&](int cls, int k, int p) {
+    const int st = p % D::NST;
+    const unsigned steps = (unsigned)min(D::CS, D::STEPS - k * D::CS);
+    bulk_load(sbase + (unsigned)D::O_ROWS + st * D::CS * 1024,
+              reinterpret_cast<const char*>(a.rows) + ((size_t)(cls - 1) * D::STEPS + (size_t)k * D::CS) * 1024,
+              steps * 1024, bar0 + 8 * st);
+  };
+  // class of row m of a block (node m of the halo order, seen from the tile)
+  auto row_class = [&](int m) {
+    const int l0 = m % D::HX, l1 = DIM == 3 ? (m / D::HX) % D::HY : m / D::HX, l2 = DIM == 3 ? m / (D::HX * D::HY) : 0;
+    if (l0 >= D::TX || l1 >= D::TY || l2 >= D::TZ) return 0;
+    return scls[(l0 + R) + D::HX * ((l1 + R) + (DIM == 3 ? D::HY * (l2 + R) : 0))] & 3;
+  };
+#pragma unroll
+  for (int q = 0; q < NH; ++q)
+    if (q * D::THREADS + tid < D::NHALO) scls[q * D::THREADS + tid] = hc[q];
+  __syncthreads();
+  // ---- largest exponent of the values per class
+  int em0 = -100000, em1 = -100000;
+#pragma unroll
+  for (int q = 0; q < NH; ++q) {
+    const int tag = hc[q] >> 2;
+    if (tag != 1 && tag != 2) continue;
+#pragma unroll
+    for (int c = 0; c < ND; ++c) {
+      const int e = (__double2hiint(hv[q][c]) >> 20) & 0x7ff;
+      if (e == 0x7ff) sbad = 1;
+      const int ee = e == 0 ? -100000 : e + (c == DIM ? delta[tag - 1] : 0);
+      if (tag == 1) em0 = max(em0, ee);
+      else em1 = max(em1, ee);
+    }
+  }
+  em0 = __reduce_max_sync(0xffffffffu, em0);
+  em1 = __reduce_max_sync(0xffffffffu, em1);
+  if (lane == 0) {
+    if (em0 > -100000) atomicMax(&semax[0], em0);
+    if (em1 > -100000) atomicMax(&semax[1], em1);
+  }
+  // ---- blocks that hold nodes of a class; a thread's own nodes: row tid %
+  // 128 of every second block
+  constexpr int NB = (D::NBLK + 1) / 2;
+  int rc[NB];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) {
+    const int blk = 2 * q + (wib >> 2);
+    rc[q] = blk < D::NBLK ? row_class(blk * 128 + (wib & 3) * 32 + lane) : 0;
+    const unsigned b1 = __ballot_sync(0xffffffffu, rc[q] == 1), b2 = __ballot_sync(0xffffffffu, rc[q] == 2);
+    if (lane == 0) {
+      if (b1) atomicOr(&sblk[0], 1u << blk);
+      if (b2) atomicOr(&sblk[1], 1u << blk);
+    }
+  }
+  __syncthreads();
+  if ((sblk[0] | sblk[1]) == 0u) return;
+  auto usable = [&](int cls) {
+    const int em = semax[cls - 1];
+    return !sbad && sc_ok[cls - 1] && (em == -100000 || (em >= 1022 - 500 && em <= 1022 + 500));
+  };
+  // ---- W of the first class on its way while the digits are written
+  const int first = sblk[0] ? 1 : 2;
+  if (tid == 0 && usable(first))
+    for (int k = 0; k < D::NST && k < D::NCH; ++k) load_w(first, k, k);
+  if (wib == 1) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(&stmem);
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(at), "n"(D::TMEM) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // ---- digits; zeros where no product reads a value
+#pragma unroll
+  for (int q = 0; q < NH; ++q) {
+    const int tag = hc[q] >> 2, n = q * D::THREADS + tid;
+    if (n >= D::NHALO) continue;
+#pragma unroll
+    for (int c = 0; c < ND; ++c) {
+      uint4 dg = make_uint4(0u, 0u, 0u, 0u);
+      if (tag == 1 || tag == 2) dg = digits_of(fixed_point(hv[q][c], semax[tag - 1], c == DIM ? delta[tag - 1] : 0));
+      *reinterpret_cast<uint4*>(smem + ((size_t)c * D::PLANE + n) * 16) = dg;
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = stmem;
+  int piece = 0;  // pieces of W so far: parities of their barriers
+  unsigned done = 0;
+  for (int cls = 1; cls <= 2; ++cls) {
+    const unsigned blocks = sblk[cls - 1];
+    if (blocks == 0u) continue;
+    const int em = semax[cls - 1];
+    const bool zero = em == -100000;
+    const bool plain = sfail || !usable(cls);
+    if (!plain) {
+      if (wib == 0) {
+        if (elect_one()) {
+          // ---- one thread: the products of each piece of W for every block.
+          // Descriptors: no swizzle, core matrices of 8 rows x 16 bytes; left
+          // operand: rows 16 bytes apart, groups of 8 rows 128; right: the
+          // halves of K 512 bytes apart, the columns' groups 128
+          const unsigned long long hi = ((unsigned long long)(128 >> 4) << 32) | (1ull << 46);
+          const unsigned idesc = (1u << 4) | ((unsigned)(D::N >> 3) << 17) | ((128u >> 4) << 24);
+          const unsigned a0 = sbase >> 4;
+          bool ok = true;
+          int loaded = cls == first ? (D::NST < D::NCH ? D::NST : D::NCH) : 0;
+          for (; loaded < D::NST && loaded < D::NCH; ++loaded) {
+            const int p = piece + loaded;
+            if (p >= D::NST)
+              ok = ok && mbar_wait(bar0 + 8 * (D::NST + p % D::NST), (unsigned)((p / D::NST - 1) & 1));
+            if (!ok) break;
+            load_w(cls, loaded, p);
+          }
+          for (int k = 0; k < D::NCH; ++k) {
+            const int p = piece + k, st = p % D::NST;
+            if (k > 0 && k - 1 + D::NST < D::NCH) {
+              // the piece before has been issued; when its products are done its place takes another
+              const int u = p - 1;
+              ok = ok && mbar_wait(bar0 + 8 * (D::NST + u % D::NST), (unsigned)((u / D::NST) & 1));
+              if (ok) {
+                load_w(cls, loaded, piece + loaded);
+                ++loaded;
+              }
+            }
+            ok = ok && mbar_wait(bar0 + 8 * st, (unsigned)((p / D::NST) & 1));
+            if (!ok) break;
+            tc_fence_after();
+            const unsigned b0 =
+                ((sbase + (unsigned)D::O_ROWS + st * D::CS * 1024) >> 4) | ((512u >> 4) << 16);
+            const int t0 = k * D::CS, t1 = min(t0 + D::CS, D::STEPS);
+            // A product reads 4 KB of digits and 1 KB of W at 128 bytes a
+            // clock: 40 clocks.  W in one piece: block by block, so that the
+            // results of one are taken while the next runs
+            if (D::NCH == 1) {
+#pragma unroll
+              for (int blk = 0; blk < D::NBLK; ++blk) {
+                if ((blocks >> blk) & 1u) {
+#pragma unroll 6
+                  for (int t = 0; t < D::STEPS; ++t)
+                    tc_mma(tmem + blk * D::N, hi | (unsigned long long)(soffs[t] + (a0 + blk * 128)),
+                           hi | (unsigned long long)(b0 + (unsigned)t * 64), idesc, t > 0);
+                }
+                tc_commit(bar_done + 8 * blk);
+              }
+              tc_commit(bar0 + 8 * (D::NST + st));
+            } else {
+              unsigned so = soffs[t0] + a0;
+#pragma unroll 2
+              for (int t = t0; t < t1; ++t) {
+                const unsigned next = soffs[t + 1 < t1 ? t + 1 : t] + a0;
+                const unsigned long long db = hi | (unsigned long long)(b0 + (unsigned)(t - t0) * 64);
+#pragma unroll
+                for (int blk = 0; blk < D::NBLK; ++blk)
+                  if ((blocks >> blk) & 1u)
+                    tc_mma(tmem + blk * D::N, hi | (unsigned long long)(so + blk * 128), db, idesc, t > 0);
+                so = next;
+              }
+              tc_commit(bar0 + 8 * (D::NST + st));
+            }
+          }
+          if (D::NCH > 1) tc_commit(bar_done);
+          if (!ok) {
+            // give up: once more for the copies on their way; what waits for
+            // the products waits no longer than its own limit
+            sfail = 1;
+            for (int k = loaded > D::NST ? loaded - D::NST : 0; k < loaded; ++k)
+              mbar_wait(bar0 + 8 * ((piece + k) % D::NST), (unsigned)(((piece + k) / D::NST) & 1));
+          }
+        }
+        __syncwarp();
+      }
+      piece += D::NCH;
+    }
+    // ---- what the thread's nodes bring besides the product, loaded meanwhile
+    double own[NB][ND];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      if (rc[q] != cls) continue;
+      const int m = (2 * q + (wib >> 2)) * 128 + (wib & 3) * 32 + lane;
+      const int i = bx + m % D::HX, j = by + (DIM == 3 ? (m / D::HX) % D::HY : m / D::HX);
+      const int k = DIM == 3 ? bz + m / (D::HX * D::HY) : 0;
+      const long long n = i + (long long)g.nn[0] * (j + (long long)(DIM == 3 ? g.nn[1] : 1) * k);
+      const double* from = KIND == 0 ? a.x : a.b;
+#pragma unroll
+      for (int c = 0; c < ND; ++c) own[q][c] = from ? from[n * ND + c] : 0.0;
+    }
+    double scale[ND];
+#pragma unroll
+    for (int n = 0; n < ND; ++n) {
+      scale[n] = plain ? 1.0 : zero ? 0.0 : pow2(a.sc[cls - 1].rowexp[n] + (em - 1022) - 36);
+      if (KIND == 0) scale[n] = a.omega * scale[n];
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int blk = 2 * q + (wib >> 2);
+      if (blk >= D::NBLK || !((blocks >> blk) & 1u)) continue;
+      const int m = blk * 128 + (wib & 3) * 32 + lane;
+      const int ia[3] = {bx + m % D::HX, by + (DIM == 3 ? (m / D::HX) % D::HY : m / D::HX),
+                         DIM == 3 ? bz + m / (D::HX * D::HY) : 0};
+      double y[ND];
+      bool fp64 = plain;
+      if (!fp64 && !mbar_wait(bar_done + 8 * (NDONE > 1 ? blk : 0), done & 1)) {
+        fp64 = true;  // no products: say so and form them in FP64
+        if (lane == 0) {
+          atomicOr(a.err, kErrTimeout);
+          sfail = 1;
+        }
+#pragma unroll
+        for (int n = 0; n < ND; ++n) scale[n] = KIND == 0 ? a.omega : 1.0;
+      }
+      if (fp64) {
+        if (rc[q] == cls) fp64_product<DIM, KIND>(g, a.w + (size_t)(cls - 1) * D::NSLOT * ND, a.v, ia, y);
+      } else {
+        tc_fence_after();
+        unsigned v[32];
+        tc_load32(tmem + ((unsigned)(wib & 3) << 21) + blk * D::N, v);
+#pragma unroll
+        for (int n = 0; n < ND; ++n) {
+          // hi = S_0 2^24 + S_1 2^16 + S_2 2^8 + S_3, lo likewise of S_4..S_7
+          long long h[2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const unsigned* S = v + n * 8 + k * 4;
+            const int s0 = __float2int_rn(__uint_as_float(S[0])), s1 = __float2int_rn(__uint_as_float(S[1]));
+            const int s2 = __float2int_rn(__uint_as_float(S[2])), s3 = __float2int_rn(__uint_as_float(S[3]));
+            h[k] = (((long long)s0 * 256 + s1) << 16) + ((long long)s2 * 256 + s3);
+          }
+          // hi + lo 2^-32 without integer conversions (both below 2^51)
+          y[n] = (__longlong_as_double(0x4338000000000000ll + h[0]) - (6755399441055744.0 + 1572864.0)) +
+                 __longlong_as_double(0x4138000000000000ll + h[1]);
+        }
+      }
+      if (rc[q] == cls) store_product<DIM, KIND>(g, a, ia, own[q], y, scale);
+    }
+    if (!plain) done ^= 1;
+    if (cls == 1 && sblk[1] != 0u) {  // the accumulators are read before the other class's products
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (wib == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(D::TMEM) : "memory");
+}
+
+// ---- plan ------------------------------------------------------------------
+
+// base class of a node's product: the class of the node's cells where the
+// whole box is in the grid, unconstrained and of that class (KIND 0: node
+// classes over the 5^d box; KIND 1: the node's own class, free neighbours)
+template <int DIM, int KIND>
+__global__ void digit_class_kernel(LevelGeom g, const unsigned char* __restrict__ nclass,
+                                   const unsigned char* __restrict__ mask, unsigned char* __restrict__ cls,
+                                   int* __restrict__ rep) {
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (unsigned)g.nnodes) return;
+  int ia[3];
+  decode_node<DIM>(g, i, ia);
+  constexpr int R = Dig<DIM, KIND>::R, RZ = DIM == 3 ? R : 0;
+  int c = nclass[i];
+  for (int dz = -RZ; dz <= RZ && c; ++dz)
+    for (int dy = -R; dy <= R && c; ++dy)
+      for (int dx = -R; dx <= R && c; ++dx) {
+        const int b0 = ia[0] + dx, b1 = ia[1] + dy, b2 = ia[2] + dz;
+        if (b0 < 0 || b0 > g.n[0] || b1 < 0 || b1 > g.n[1] || (DIM == 3 && (b2 < 0 || b2 > g.n[2]))) { c = 0; break; }
+        const long long bn = b0 + (long long)g.nn[0] * (b1 + (long long)g.nn[1] * b2);
+        if (mask[bn] & 7) c = 0;
+        if (KIND == 0 && nclass[bn] != nclass[i]) c = 0;
+      }
+  cls[i] = (unsigned char)c;
+  if (c) atomicMin(&rep[c], (int)i);
+}
+
+// KIND 1: a node whose stencil is not the representative's is no class node
+template <int DIM>
+__global__ void digit_compare_kernel(LevelGeom g, const double* __restrict__ st, unsigned char* __restrict__ cls,
+                                     const int* __restrict__ rep) {
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (unsigned)g.nnodes) return;
+  const int c = cls[i];
+  if (!c) return;
+  const int r = rep[c];
+  constexpr int N = (DIM == 3 ? 27 : 9) * (2 * DIM + 2);
+  bool same = true;
+  for (int t = 0; t < N; ++t) same = same && st[(long long)t * g.nnodes + i] == st[(long long)t * g.nnodes + r];
+  if (!same) cls[i] = 0;
+}
+
+// bits 2-3: classes of the products that read the node
+template <int DIM, int KIND>
+__global__ void digit_tag_kernel(LevelGeom g, const unsigned char* __restrict__ in, unsigned char* __restrict__ out) {
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (unsigned)g.nnodes) return;
+  int ia[3];
+  decode_node<DIM>(g, i, ia);
+  constexpr int R = Dig<DIM, KIND>::R, RZ = DIM == 3 ? R : 0;
+  int tag = 0;
+  for (int dz = -RZ; dz <= RZ; ++dz)
+    for (int dy = -R; dy <= R; ++dy)
+      for (int dx = -R; dx <= R; ++dx) {
+        const int b0 = ia[0] + dx, b1 = ia[1] + dy, b2 = ia[2] + dz;
+        if (b0 < 0 || b0 > g.n[0] || b1 < 0 || b1 > g.n[1] || (DIM == 3 && (b2 < 0 || b2 > g.n[2]))) continue;
+        const int c = in[b0 + (long long)g.nn[0] * (b1 + (long long)g.nn[1] * b2)] & 3;
+        if (c) tag |= 1 << (c - 1);
+      }
+  out[i] = (unsigned char)((in[i] & 3) | (tag << 2));
+}
+
+// products that read a node tagged by both classes leave the digits; counts
+// the nodes that stay (count[0]) and marks the classes that are left (count[1])
+template <int DIM, int KIND>
+__global__ void digit_settle_kernel(LevelGeom g, const unsigned char* __restrict__ in, unsigned char* __restrict__ out,
+                                    int* __restrict__ count) {
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  int c = 0;
+  if (i < (unsigned)g.nnodes) {
+    int ia[3];
+    decode_node<DIM>(g, i, ia);
+    constexpr int R = Dig<DIM, KIND>::R, RZ = DIM == 3 ? R : 0;
+    c = in[i] & 3;
+    for (int dz = -RZ; dz <= RZ && c; ++dz)
+      for (int dy = -R; dy <= R && c; ++dy)
+        for (int dx = -R; dx <= R && c; ++dx)
+          if ((in[(ia[0] + dx) + (long long)g.nn[0] * ((ia[1] + dy) + (long long)g.nn[1] * (ia[2] + dz))] >> 2) == 3)
+            c = 0;
+    out[i] = (unsigned char)((in[i] & ~3) | c);
+  }
+  const int n = __popc(__ballot_sync(0xffffffffu, c != 0));
+  if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, n);
+  if (c) atomicOr(count + 1, 1 << c);
+}
+
+// the nodes without a class, in order
+constexpr int kListBlock = 1024;
+__global__ void digit_list_count_kernel(int n, const unsigned char* __restrict__ cls, int* __restrict__ counts) {
+  __shared__ int sm;
+  if (threadIdx.x == 0) sm = 0;
+  __syncthreads();
+  const int i = blockIdx.x * kListBlock + threadIdx.x;
+  const int f = __popc(__ballot_sync(0xffffffffu, i < n && !(cls[i] & 3)));
+  if ((threadIdx.x & 31) == 0) atomicAdd(&sm, f);
+  __syncthreads();
+  if (threadIdx.x == 0) counts[blockIdx.x] = sm;
+}
+// exclusive scan by one CTA
+__global__ void __launch_bounds__(1024) digit_list_scan_kernel(int nb, int* __restrict__ counts) {
+  __shared__ int sm[32];
+  int run = 0;
+  for (int b0 = 0; b0 < nb; b0 += 1024) {
+    const int b = b0 + threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c = b < nb ? counts[b] : 0;
+    int s = c;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += t;
+    }
+    if (lane == 31) sm[w] = s;
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int k = 0; k < 32; ++k) {
+      if (k < w) before += sm[k];
+      total += sm[k];
+    }
+    if (b < nb) counts[b] = run + before + s - c;
+    run += total;
+    __syncthreads();
+  }
+}
+__global__ void digit_list_place_kernel(int n, const unsigned char* __restrict__ cls, const int* __restrict__ offs,
+                                        int* __restrict__ list) {
+  __shared__ int sm[32];
+  const int i = blockIdx.x * kListBlock + threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool f = i < n && !(cls[i] & 3);
+  const unsigned bal = __ballot_sync(0xffffffffu, f);
+  if (lane == 0) sm[w] = __popc(bal);
+  __syncthreads();
+  int before = offs[blockIdx.x];
+  for (int k = 0; k < w; ++k) before += sm[k];
+  if (f) list[before + __popc(bal & ((1u << lane) - 1u))] = i;
+}
+
+// W of a class in slot order (CTA per class): the representative's cached
+// rows or stencil; then scales and the right operand.
+template <int DIM, int KIND>
+__global__ void __launch_bounds__(256)
+    digit_rows_kernel(LevelGeom g, const double* __restrict__ src, const int* __restrict__ prow,
+                      const int* __restrict__ rep, double* __restrict__ w, uint4* __restrict__ rows,
+                      DigitScale* __restrict__ sc) {
+  using D = Dig<DIM, KIND>;
+  constexpr int ND = D::ND, NSLOT = D::NSLOT;
+  const int c = blockIdx.x, tid = threadIdx.x;
+  const int i = rep[c + 1];
+  __shared__ int smax[4 + 2], sok;
+  __shared__ int sdig[4][8];  // sum over the slots of |digit|
+  double* W = w + (size_t)c * NSLOT * ND;
+  if (tid < 6) smax[tid] = -100000;
+  if (tid < 32) sdig[tid / 8][tid % 8] = 0;
+  if (tid == 0) sok = 1;
+  __syncthreads();
+  if (i == 0x7fffffff) {  // no node of this class
+    if (tid == 0) {
+      for (int r = 0; r < 4; ++r) sc[c].rowexp[r] = 0;
+      sc[c].delta = 0;
+      sc[c].ok = 0;
+    }
+    return;
+  }
+  for (int t = tid; t < NSLOT * ND; t += blockDim.x) {
+    const int j = t / ND, r = t % ND;
+    int o[3], k, at;
+    slot_of<DIM, KIND>(j, o, &k, &at);
+    double v;
+    if (KIND == 0) {
+      const int pr = prow[i];
+      v = src[((size_t)(pr < 0 ? -pr - 1 : pr) * NSLOT + at) * ND + r];
+    } else {
+      constexpr int SP = 2 * DIM + 2;
+      const int nb = at / ND;
+      int e = -1;  // velocity components do not couple
+      if (r < DIM) e = k == r ? 0 : (k == DIM ? 1 + r : -1);
+      else e = k < DIM ? 1 + DIM + k : 1 + 2 * DIM;
+      v = e >= 0 ? src[((long long)nb * SP + e) * g.nnodes + i] : 0.0;
+    }
+    W[t] = v;
+    const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    if (e == 0x7ff) sok = 0;
+    if (e != 0 && (r < DIM) == (k < DIM)) atomicMax(&smax[r < DIM ? 4 : 5], e);
+  }
+  __syncthreads();
+  const int eu = smax[4], ep = smax[5];
+  const int d2 = eu > -100000 && ep > -100000 ? ep - eu : 0;
+  const int delta = (d2 + (d2 < 0 ? -1 : 1)) / 2;
+  for (int t = tid; t < NSLOT * ND; t += blockDim.x) {
+    int o[3], k, at;
+    slot_of<DIM, KIND>(t / ND, o, &k, &at);
+    const int e = (__double2hiint(W[t]) >> 20) & 0x7ff;
+    if (e != 0) atomicMax(&smax[t % ND], e - (k == DIM ? delta : 0));
+  }
+  __syncthreads();
+  // right operand: per slot and row the 8 x 8 block [d][s] = w_{d-s}, stored
+  // [step][slot of the pair][row][d][s]
+  uint4* out = rows + (size_t)c * D::STEPS * 64;
+  for (int t = tid; t < D::STEPS * 64; t += blockDim.x) {
+    const int slot = t / 32, r = (t / 8) % 4, d = t % 8;
+    unsigned v[4] = {0u, 0u, 0u, 0u};
+    if (slot < NSLOT && r < ND) {
+      int o[3], k, at;
+      slot_of<DIM, KIND>(slot, o, &k, &at);
+      const uint4 dg = digits_of(fixed_point(W[(size_t)slot * ND + r], smax[r], k == DIM ? -delta : 0));
+      const unsigned h[4] = {dg.x, dg.y, dg.z, dg.w};
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int j = d - s;
+        unsigned x = 0u;
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+          if (j == m) x = (m & 1) ? h[m / 2] >> 16 : h[m / 2] & 0xffffu;
+        v[s / 2] |= x << (16 * (s & 1));
+        if (s == 0) atomicAdd(&sdig[r][d], abs((int)__half2float(__ushort_as_half((unsigned short)x))));
+      }
+    }
+    out[t] = make_uint4(v[0], v[1], v[2], v[3]);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int r = 0; r < 4; ++r) {
+      const int e = r < ND && smax[r] > -100000 ? smax[r] - 1022 : 0;
+      if (e < -400 || e > 400) sok = 0;
+      sc[c].rowexp[r] = e;
+      // |S_d| <= sum over s <= d of (sum |w_s|) max |v_{d-s}|; a leading digit is at most 64
+      for (int d = 0; d <= 5; ++d) {
+        long long b = 0;
+        for (int s = 0; s <= d; ++s) b += (long long)sdig[r][s] * (s == d ? 64 : 128);
+        if (b >= (1 << 24)) sok = 0;
+      }
+    }
+    if (delta < -200 || delta > 200) sok = 0;
+    sc[c].delta = delta;
+    sc[c].ok = sok;
+  }
+}
+
+template <int DIM, int KIND>
+cudaError_t run_product(const LevelGeom& g, const DigitPlan& p, DigArgs a, cudaStream_t s) {
+  using D = Dig<DIM, KIND>;
+  a.cls = p.cls;
+  a.rows = p.rows;
+  a.w = p.w;
+  a.sc = p.sc;
+  a.err = p.err;
+  a.list = p.list;
+  a.nlist = (int)p.nlist;
+  a.list_blocks = DIM == 2 ? (int)((p.nlist + 63) / 64) : 0;  // 4 lanes a node
+  auto kern = digit_product_kernel<DIM, KIND>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D::BYTES);
+  if (e != cudaSuccess) return e;
+  const int tx = (g.nn[0] - 2 * D::R + D::TX - 1) / D::TX, ty = (g.nn[1] - 2 * D::R + D::TY - 1) / D::TY;
+  const int tz = DIM == 3 ? (g.nn[2] - 2 * D::R + D::TZ - 1) / D::TZ : 1;
+  const unsigned blocks = (unsigned)a.list_blocks + (unsigned)tx * ty * tz;
+  kern<<<blocks, D::THREADS, D::BYTES, s>>>(g, a, tx, ty);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+template <int DIM, int KIND>
+cudaError_t build_plan(const LevelGeom& g, const double* src, const unsigned char* nclass, const unsigned char* mask,
+                       const int* prow, DigitPlan* p, unsigned char* tmp, int* rep, int* counts, cudaStream_t s) {
+  using D = Dig<DIM, KIND>;
+  const unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
+  const int n = (int)g.nnodes, nb = (n + kListBlock - 1) / kListBlock;
+  // rep[1], rep[2]: representatives; rep[4]: class nodes, rep[5]: classes
+  const int init[6] = {0x7fffffff, 0x7fffffff, 0x7fffffff, 0, 0, 0};
+  cudaError_t e = cudaMemcpyAsync(rep, init, sizeof(init), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  digit_class_kernel<DIM, KIND><<<blocks, 256, 0, s>>>(g, nclass, mask, p->cls, rep);
+  if (KIND == 1) digit_compare_kernel<DIM><<<blocks, 256, 0, s>>>(g, src, p->cls, rep);
+  digit_tag_kernel<DIM, KIND><<<blocks, 256, 0, s>>>(g, p->cls, tmp);
+  digit_settle_kernel<DIM, KIND><<<blocks, 256, 0, s>>>(g, tmp, p->cls, rep + 4);
+  digit_list_count_kernel<<<nb, kListBlock, 0, s>>>(n, p->cls, counts);
+  digit_list_scan_kernel<<<1, 1024, 0, s>>>(nb, counts);
+  digit_list_place_kernel<<<nb, kListBlock, 0, s>>>(n, p->cls, counts, p->list);
+  digit_rows_kernel<DIM, KIND><<<2, 256, 0, s>>>(g, src, prow, rep, p->w, p->rows, p->sc);
+  note_launches(7 + KIND);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  int got[2] = {0, 0};
+  e = cudaMemcpyAsync(got, rep + 4, sizeof(got), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  p->nlist = g.nnodes - got[0];
+  return e;
+}
+
+}  // namespace
+
+size_t digit_plan_rows_bytes(int dim, int kind) {
+  const size_t steps = dim == 3 ? Dig<3, 0>::STEPS : kind == 0 ? Dig<2, 0>::STEPS : Dig<2, 1>::STEPS;
+  return 2 * steps * 64 * sizeof(uint4);
+}
+size_t digit_plan_w_bytes(int dim, int kind) {
+  const size_t slots = dim == 3 ? Dig<3, 0>::NSLOT : kind == 0 ? Dig<2, 0>::NSLOT : Dig<2, 1>::NSLOT;
+  return 2 * slots * (dim + 1) * sizeof(double);
+}
+int digit_plan_counts(long long nnodes) { return (int)((nnodes + kListBlock - 1) / kListBlock); }
+
+cudaError_t build_digit_plan(const LevelGeom& g, int kind, const double* src, const unsigned char* nclass,
+                             const unsigned char* mask, const int* prow, DigitPlan* p, unsigned char* tmp, int* rep,
+                             int* counts, cudaStream_t s) {
+  if (g.dim == 2)
+    return kind == 0 ? build_plan<2, 0>(g, src, nclass, mask, prow, p, tmp, rep, counts, s)
+                     : build_plan<2, 1>(g, src, nclass, mask, prow, p, tmp, rep, counts, s);
+  return build_plan<3, 0>(g, src, nclass, mask, prow, p, tmp, rep, counts, s);
+}
+
+// 3D: two launches (a tile's CTA takes most of an SM's shared memory; run
+// beside one, the FP64 products lost more to the smaller L1 than they gained)
+cudaError_t launch_digit_apply(const LevelGeom& g, const DigitPlan& p, const double* coef, const unsigned char* mask,
+                               const double* rpad, double omega, double* x, const int* prow, cudaStream_t s) {
+  DigArgs a{};
+  a.v = rpad;
+  a.x = x;
+  a.omega = omega;
+  a.coef = coef;
+  a.mask = mask;
+  a.prow = prow;
+  if (g.dim == 2) return run_product<2, 0>(g, p, a, s);
+  if (p.nlist > 0) {
+    const cudaError_t e =
+        launch_patch_apply(g, FC_PREC_FP64, coef, mask, rpad, nullptr, omega, x, prow, s, p.list, p.nlist);
+    if (e != cudaSuccess) return e;
+  }
+  return run_product<3, 0>(g, p, a, s);
+}
+
+cudaError_t launch_digit_residual(const LevelGeom& g, const DigitPlan& p, const double* st, const unsigned char* mask,
+                                  const double* x, const double* b, double* r, double* rpad, cudaStream_t s) {
+  DigArgs a{};
+  a.v = x;
+  a.b = b;
+  a.r = r;
+  a.rpad = rpad;
+  a.coef = st;
+  a.mask = mask;
+  return run_product<2, 1>(g, p, a, s);
+}
+
+}  // namespace fc

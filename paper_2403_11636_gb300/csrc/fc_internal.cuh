@@ -21,6 +21,7 @@ enum DevErr : unsigned {
   kErrSingularPatch = 2u,
   kErrSingularCoarse = 4u,
   kErrBadIndex = 8u,
+  kErrTimeout = 16u,  // a bounded wait gave up (fc_digits.cu; the products were formed in FP64)
 };
 
 struct Shape {
@@ -150,6 +151,35 @@ struct AmrLevel {
   unsigned long long rows_flop = 0;  // 2 x (patch DoFs x free owned DoFs) summed over the patches
 };
 
+// Scales of a class's rows W as digits: |w| 2^(-delta on pressure columns) <
+// 2^rowexp; ok is zero where the class is empty or W is out of range.
+struct DigitScale {
+  int rowexp[4];
+  int delta;
+  int ok;
+};
+
+// Levels of at least so many nodes get plans: below, a tile's fixed time (its
+// loads, digits and products follow one another) is more than the FP64 kernels
+// need.  GB300, us, class products / FP64 kernels: 2D patch apply 13 / 8 at
+// 65^2 nodes, 15 / 22 at 257^2, 27 / 80 at 1025 x 257, 164 / 790 at 1537^2; 2D
+// residual 13 / 5 at 65^2, 14 / 9 at 257^2, 20 / 29 at 1025 x 257, 125 / 263 at
+// 1537^2; 3D patch apply 172 + 417 (other patches) / 711 at 65^3 porous.
+constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 130000, kDigitApply3 = 100000;
+
+// Which nodes of a level take their product with the class rows on the tensor
+// cores, and those rows (fc_digits.cu).
+struct DigitPlan {
+  bool on = false;
+  unsigned char* cls = nullptr;  // per node: bits 0-1 class of its product, bits 2-3 classes of products that read it
+  int* list = nullptr;           // nodes without a class, in order
+  long long nlist = 0;
+  uint4* rows = nullptr;         // W as a tensor-core operand, [class][step][1 KB]
+  double* w = nullptr;           // W, [class][slot][row]
+  DigitScale* sc = nullptr;      // [class]
+  unsigned* err = nullptr;       // the handle's error word
+};
+
 struct Level {
   LevelGeom g;
   double* st = nullptr;         // stencil, SPN * 3^d * nnodes
@@ -200,6 +230,9 @@ struct Level {
   int nwork = 0;
   int cls_blk[2] = {-1, -1};            // stored blocks of the patch classes 1 and 2
   unsigned long long active_work = 0;   // active DoFs summed over the stored blocks
+  // class products on the tensor cores (fc_digits.cu): [0] patch apply with
+  // FP64 rows, [1] FP64 operator
+  DigitPlan dig[2];
   // Q2-Q1 variant (fc_options.element = 1, see fc_q2.cu): grid sizes, node
   // masks, stencil blocks, padded residual copies (velocity halo 4 nodes,
   // pressure halo 1 vertex); the patch rows live in coef, Dirichlet values
@@ -368,6 +401,8 @@ cudaError_t launch_cell_elements_q2(const LevelGeom& g, double* eA, double* eB, 
 cudaError_t launch_patch_classes(const LevelGeom& g, const unsigned char* cclass, const unsigned char* mask,
                                  unsigned char* nclass, int* pclass, int* rep, int* work, int* nwork,
                                  int* prow, int dedup, cudaStream_t s);
+cudaError_t launch_node_classes(const LevelGeom& g, const unsigned char* cclass, unsigned char* nclass,
+                                cudaStream_t s);
 // assembly (fc_assemble.cu)
 cudaError_t launch_assemble(const LevelGeom& g, const double* eA, const double* eB, double* st,
                             cudaStream_t s);
@@ -426,9 +461,25 @@ cudaError_t launch_patch_rows_pair(const LevelGeom& g, const double* st, const u
                                    double* coef64, unsigned* d_err, const int* work, long long nwork,
                                    const int* outidx, cudaStream_t s);
 // prow (nullable = identity) maps a patch to its stored row / factor block
+// (FP64 rows: over all patches, or, in 3D, over the nlist patches of list)
 cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coef,
                                const unsigned char* mask, const double* rpad, const float* rpad32,
-                               double omega, double* x, const int* prow, cudaStream_t s);
+                               double omega, double* x, const int* prow, cudaStream_t s,
+                               const int* list = nullptr, long long nlist = 0);
+// FP64 class products on the tensor cores (fc_digits.cu).  kind 0: patch apply
+// (src = FP64 rows), 1: operator (src = stencil; 2D).  p's arrays are allocated by
+// the caller (sizes below); tmp nnodes bytes, rep 6 ints, counts
+// digit_plan_counts ints of scratch.  Synchronises.
+size_t digit_plan_rows_bytes(int dim, int kind);
+size_t digit_plan_w_bytes(int dim, int kind);
+int digit_plan_counts(long long nnodes);
+cudaError_t build_digit_plan(const LevelGeom& g, int kind, const double* src, const unsigned char* nclass,
+                             const unsigned char* mask, const int* prow, DigitPlan* p, unsigned char* tmp, int* rep,
+                             int* counts, cudaStream_t s);
+cudaError_t launch_digit_apply(const LevelGeom& g, const DigitPlan& p, const double* coef, const unsigned char* mask,
+                               const double* rpad, double omega, double* x, const int* prow, cudaStream_t s);
+cudaError_t launch_digit_residual(const LevelGeom& g, const DigitPlan& p, const double* st, const unsigned char* mask,
+                                  const double* x, const double* b, double* r, double* rpad, cudaStream_t s);
 // cache_matrix factors of a level: band records (3D) or dense records (2D),
 // plus the dense records and node list of the 3D patches that need them
 struct FactorStore {
@@ -523,5 +574,19 @@ cudaError_t launch_mgs_fused(long long n, double* w, const double* v_prev, const
 cudaError_t launch_givens(double* small, int m, int j, double bnorm, cudaStream_t s);
 cudaError_t launch_update_x(long long n, int k, int m, const double* small, const double* Z,
                             double* x, cudaStream_t s);
+
+// the FP64 residual of a level, and the patch apply with cached rows: class
+// products on the tensor cores where the level has a plan for them
+inline cudaError_t residual_fp64(const Level& L, const double* x, const double* b, double* r, double* rpad,
+                                 cudaStream_t s) {
+  if (L.dig[1].on) return launch_digit_residual(L.g, L.dig[1], L.st, L.mask, x, b, r, rpad, s);
+  return launch_residual(L.g, L.st, L.mask, x, b, r, rpad, s);
+}
+inline cudaError_t apply_rows(const Level& L, fc_prec prec, const double* rpad, const float* rpad32, double omega,
+                              double* x, cudaStream_t s) {
+  if (prec == FC_PREC_FP64 && L.dig[0].on)
+    return launch_digit_apply(L.g, L.dig[0], (const double*)L.coef, L.mask, rpad, omega, x, L.prow, s);
+  return launch_patch_apply(L.g, prec, L.coef, L.mask, rpad, rpad32, omega, x, L.prow, s);
+}
 
 }  // namespace fc

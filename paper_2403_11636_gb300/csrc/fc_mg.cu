@@ -6,80 +6,21 @@
 
 #include <algorithm>
 
-#include "fc_internal.cuh"
+#include "fc_node.cuh"
 
 namespace fc {
 
 namespace {
 
-// ---------------------------------------------------------------------------
-// residual / apply: one thread per node, the 3^d neighbour blocks of the
-// compressed stencil; constrained rows are identity rows and constrained
-// columns are skipped (their values live in b).
-// OUT: 0 -> r (unpadded, optional) and rpad (padded, optional) in float64,
-//      1 -> rpad as float32 pairs (hi, lo), 2 -> rpad as float32.
-template <int DIM, int OUT>
+template <int DIM, int OUT, int TPP>
 __global__ void __launch_bounds__(256)
     residual_kernel(LevelGeom g, const double* __restrict__ st, const unsigned char* __restrict__ mask,
                     const double* __restrict__ x, const double* __restrict__ b,
                     double* __restrict__ r, double* __restrict__ rpad, float* __restrict__ rpadf) {
-  constexpr int NB = DIM == 3 ? 27 : 9, SP = 2 * DIM + 2, ND = DIM + 1;
-  long long node = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (node >= g.nnodes) return;
-  // 32-bit decode: 64-bit division would run on the slow FP64 pipe
-  int ia[3];
-  {
-    const unsigned u = (unsigned)node, nx = (unsigned)g.nn[0], ny = (unsigned)g.nn[1];
-    const unsigned t = u / nx;
-    ia[0] = (int)(u - t * nx);
-    ia[1] = DIM == 3 ? (int)(t % ny) : (int)t;
-    ia[2] = DIM == 3 ? (int)(t / ny) : 0;
-  }
-  double acc[ND];
-#pragma unroll
-  for (int c = 0; c < ND; ++c) acc[c] = 0.0;
-#pragma unroll
-  for (int nb = 0; nb < NB; ++nb) {
-    int ib0 = ia[0] + nb % 3 - 1, ib1 = ia[1] + (nb / 3) % 3 - 1, ib2 = DIM == 3 ? ia[2] + nb / 9 - 1 : 0;
-    if (ib0 < 0 || ib0 > g.n[0] || ib1 < 0 || ib1 > g.n[1]) continue;
-    if (DIM == 3 && (ib2 < 0 || ib2 > g.n[2])) continue;
-    long long bn = ib0 + (long long)g.nn[0] * (ib1 + (long long)g.nn[1] * ib2);
-    unsigned char mb = mask[bn];
-    double xb[ND];
-#pragma unroll
-    for (int c = 0; c < ND; ++c) xb[c] = x[bn * ND + c];
-#pragma unroll
-    for (int c = 0; c < DIM; ++c)
-      if ((mb >> c) & 1) xb[c] = 0.0;
-    const double* s = st + (long long)nb * SP * g.nnodes + node;
-    double vA = s[0];
-#pragma unroll
-    for (int c = 0; c < DIM; ++c) {
-      acc[c] = acc[c] + vA * xb[c];
-      acc[c] = acc[c] + s[(1 + c) * g.nnodes] * xb[DIM];
-    }
-#pragma unroll
-    for (int c = 0; c < DIM; ++c) acc[DIM] = acc[DIM] + s[(1 + DIM + c) * g.nnodes] * xb[c];
-    acc[DIM] = acc[DIM] + s[(1 + 2 * DIM) * g.nnodes] * xb[DIM];
-  }
-  unsigned char ma = mask[node];
-  long long pn = pad_node(g, ia[0], ia[1], ia[2]);
-#pragma unroll
-  for (int c = 0; c < ND; ++c) {
-    double y = (c < DIM && ((ma >> c) & 1)) ? x[node * ND + c] : acc[c];
-    double v = b ? b[node * ND + c] - y : y;
-    if (OUT == 0) {
-      if (r) r[node * ND + c] = v;
-      if (rpad) rpad[pn * ND + c] = v;
-    } else if (OUT == 1) {
-      float hi = (float)v;
-      float lo = (float)(v - (double)hi);
-      rpadf[(pn * ND + c) * 2 + 0] = hi;
-      rpadf[(pn * ND + c) * 2 + 1] = lo;
-    } else {
-      rpadf[pn * ND + c] = (float)v;
-    }
-  }
+  const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPP;
+  const bool valid = t < g.nnodes;
+  if (TPP == 1 && !valid) return;
+  residual_node<DIM, OUT, TPP>(g, st, mask, x, b, r, rpad, rpadf, valid ? t : g.nnodes - 1, valid);
 }
 
 // ---------------------------------------------------------------------------
@@ -743,12 +684,24 @@ inline unsigned grid_for(long long n, int bs) {
 
 }  // namespace
 
+constexpr long long kResidualGroup3 = 152 * 512, kResidualGroup2 = 152 * 256;
+
 cudaError_t launch_residual(const LevelGeom& g, const double* st, const unsigned char* mask,
                             const double* x, const double* b, double* r, double* rpad,
                             cudaStream_t s) {
-  unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
-  if (g.dim == 2) residual_kernel<2, 0><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
-  else residual_kernel<3, 0><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
+  // lanes per node: one where the level fills the GPU with threads, a group on
+  // smaller levels, where a thread alone walks its neighbours' loads in turn
+  // (GB300, us, 1 lane / a group: 3D 45 / 17 at 17^3 nodes, 51 / 30 at 33^3,
+  // 139 / 150 at 65^3; 2D 6.9 / 4.6 at 33^2)
+  const int tpp = g.dim == 3 ? (g.nnodes < kResidualGroup3 ? 8 : 1) : (g.nnodes < kResidualGroup2 ? 4 : 1);
+  const unsigned blocks = (unsigned)((g.nnodes * tpp + 255) / 256);
+  if (g.dim == 2) {
+    if (tpp == 1) residual_kernel<2, 0, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
+    else residual_kernel<2, 0, 4><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
+  } else {
+    if (tpp == 1) residual_kernel<3, 0, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
+    else residual_kernel<3, 0, 8><<<blocks, 256, 0, s>>>(g, st, mask, x, b, r, rpad, nullptr);
+  }
   note_launches(1);
   return cudaGetLastError();
 }
@@ -756,8 +709,8 @@ cudaError_t launch_residual(const LevelGeom& g, const double* st, const unsigned
 cudaError_t launch_residual_df(const LevelGeom& g, const double* st, const unsigned char* mask,
                                const double* x, const double* b, float* rpad2, cudaStream_t s) {
   unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
-  if (g.dim == 2) residual_kernel<2, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad2);
-  else residual_kernel<3, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad2);
+  if (g.dim == 2) residual_kernel<2, 1, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad2);
+  else residual_kernel<3, 1, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad2);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -765,8 +718,8 @@ cudaError_t launch_residual_df(const LevelGeom& g, const double* st, const unsig
 cudaError_t launch_residual_f32(const LevelGeom& g, const double* st, const unsigned char* mask,
                                 const double* x, const double* b, float* rpad, cudaStream_t s) {
   unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
-  if (g.dim == 2) residual_kernel<2, 2><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
-  else residual_kernel<3, 2><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
+  if (g.dim == 2) residual_kernel<2, 2, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
+  else residual_kernel<3, 2, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
   note_launches(1);
   return cudaGetLastError();
 }

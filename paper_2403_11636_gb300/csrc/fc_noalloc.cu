@@ -98,10 +98,10 @@ extern "C" fc_status fc_smooth_noalloc(fc_handle h, int level, double* x, const 
   for (int s = 0; s < nsweeps; ++s) {
     if (inverse && prec == FC_PREC_DF64) e = launch_residual_df(L.g, L.st, L.mask, x, b, rpadf, h->stream);
     else if (inverse && prec != FC_PREC_FP64) e = launch_residual_f32(L.g, L.st, L.mask, x, b, rpadf, h->stream);
-    else e = launch_residual(L.g, L.st, L.mask, x, b, nullptr, rpad, h->stream);
+    else e = residual_fp64(L, x, b, nullptr, rpad, h->stream);
     if (e != cudaSuccess) return fail(h, FC_ERR_CUDA, cudaGetErrorString(e));
     if (inverse)
-      e = launch_patch_apply(L.g, prec, L.coef, L.mask, rpad, rpadf, h->opt.omega, x, L.prow, h->stream);
+      e = apply_rows(L, prec, rpad, rpadf, h->opt.omega, x, h->stream);
     else if (h->opt.cache == FC_CACHE_MATRIX)
       e = launch_factor_apply(L.g, L.st, factor_store(L), L.mask, rpad, h->opt.omega, x, L.prow, h->stream);
     else

@@ -27,7 +27,7 @@
 
 #include <algorithm>
 
-#include "fc_internal.cuh"
+#include "fc_node.cuh"
 
 namespace fc {
 
@@ -1047,46 +1047,6 @@ __global__ void dense_list_kernel(long long nnodes, const int* __restrict__ prow
 // residual offset table is built once per block in shared memory, and the
 // node index is decoded in 32-bit arithmetic (64-bit division would run on
 // the FP64 pipe, 1/70 of the FP32 rate on this part).
-// Row loads: rows shared by a class of patches stay in the caches; a
-// patch's own rows are read once per sweep and streamed past L2.
-template <typename V>
-__device__ __forceinline__ V ldrow(const V* p, bool cached) {
-  return cached ? __ldg(p) : __ldcs(p);
-}
-
-template <int DIM>
-__device__ __forceinline__ void slot_table(const LevelGeom& g, int* soff) {
-  constexpr int NU = PatchDims<DIM>::NU, ND = DIM + 1, NSLOT = PatchDims<DIM>::NSLOT;
-  const int px = g.nn[0] + 4, py = g.nn[1] + 4;
-  for (int j = threadIdx.x; j < NSLOT; j += blockDim.x) {
-    int o[3], c;
-    if (j < NU * DIM) {
-      vel_off<DIM>(j / DIM, o);
-      c = j % DIM;
-    } else {
-      prs_off<DIM>(j - NU * DIM, o);
-      c = DIM;
-    }
-    soff[j] = (o[0] + px * (o[1] + py * o[2])) * ND + c;
-  }
-  __syncthreads();
-}
-
-template <int DIM>
-__device__ __forceinline__ void decode_node(const LevelGeom& g, unsigned i, int* ia) {
-  const unsigned nx = (unsigned)g.nn[0], ny = (unsigned)g.nn[1];
-  unsigned t = i / nx;
-  ia[0] = (int)(i - t * nx);
-  if (DIM == 3) {
-    unsigned u = t / ny;
-    ia[1] = (int)(t - u * ny);
-    ia[2] = (int)u;
-  } else {
-    ia[1] = (int)t;
-    ia[2] = 0;
-  }
-}
-
 template <int DIM>
 __device__ __forceinline__ void finish_update(const LevelGeom& g, long long i, const int* ia,
                                               const unsigned char* mask, const double* rc,
@@ -1100,138 +1060,19 @@ __device__ __forceinline__ void finish_update(const LevelGeom& g, long long i, c
   x[i * ND + DIM] = x[i * ND + DIM] + omega * y[DIM];
 }
 
-// Restricted prolongation R~_i^T for the apply kernels: lane c < d+1
-// updates component c of node i from the warp-reduced y (all lanes hold the
-// sums); constrained velocity components take the residual (identity row).
-// x2, when given, receives the (hi, lo) float pair of the new value.
-template <int ND>
-__device__ __forceinline__ void owned_update(unsigned i, int lane, const unsigned char* mask, double rcv,
-                                             double yv, double omega, double* x, float2* x2) {
-  if (lane >= ND) return;
-  const int c = lane;
-  const size_t k = (size_t)i * ND + c;
-  const bool fixed = c < ND - 1 && ((mask[i] >> c) & 1);
-  const double nv = x[k] + (fixed ? rcv : omega * yv);
-  x[k] = nv;
-  if (x2) {
-    float hi = (float)nv;
-    x2[k] = make_float2(hi, (float)(nv - (double)hi));
-  }
-}
-
-template <int N, typename T>
-__device__ __forceinline__ T pick(const T* v, int c) {
-  T r = v[0];
-#pragma unroll
-  for (int k = 1; k < N; ++k)
-    if (c == k) r = v[k];
-  return r;
-}
-
-
-template <int DIM, int TPP>
+// over all patches, or (LIST) over the `nlist` patches of `list`
+template <int DIM, int TPP, bool LIST>
 __global__ void __launch_bounds__(256)
     apply_fp64_kernel(LevelGeom g, const double* __restrict__ coef, const unsigned char* __restrict__ mask,
                       const double* __restrict__ rpad, double omega, double* __restrict__ x,
-                      const int* __restrict__ prow) {
-  using P = PatchDims<DIM>;
-  constexpr int ND = P::ND, NSLOT = P::NSLOT;
-  __shared__ int soff[NSLOT];
+                      const int* __restrict__ prow, const int* __restrict__ list, unsigned nlist) {
+  __shared__ int soff[SlotDims<DIM>::NSLOT];
   slot_table<DIM>(g, soff);
-  // a group of TPP lanes per patch; groups past the last patch still take
-  // part in the shuffles of their warp
-  const int lane = threadIdx.x % TPP;
+  const unsigned n = LIST ? nlist : (unsigned)g.nnodes;
   const unsigned gi = (unsigned)(((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) / TPP);
-  const bool valid = gi < (unsigned)g.nnodes;
-  const unsigned i = valid ? gi : (unsigned)g.nnodes - 1;
-  int ia[3];
-  decode_node<DIM>(g, i, ia);
-  const long long pbase = pad_node(g, ia[0], ia[1], ia[2]);
-  const double* rp = rpad + pbase * ND;
-  const int pr = prow ? prow[i] : (int)i;
-  const bool shared_rows = pr < 0;  // class rows: read through the cache
-  const double* cf = coef + (size_t)(shared_rows ? -pr - 1 : pr) * NSLOT * ND;
-  double y[4] = {0.0, 0.0, 0.0, 0.0};  // 2D: y[3] stays zero
-  // Live velocity slots.  Slots of out-of-grid nodes and of wall layers
-  // (every velocity component constrained) have zero coefficients; in 3D the
-  // 5 x 5 x 5 velocity box is clipped per direction to its live layers
-  // [x0, x1] x [y0, y1] x [z0, z1]: a patch walks rows of rx = 3 (x1 - x0 + 1)
-  // contiguous slots (a y row of a z-plane holds 15), ny rows per z-plane,
-  // nz planes, then its 3^d pressure slots.  Patches of a warp are
-  // consecutive nodes of an x row and mostly share the clipping.
-  int nv = P::NU * DIM, rx = nv, ny = 1, vbase = 0;  // unclipped: one run of all velocity slots
-  if (DIM == 3 && g.dead_layer) {
-    const unsigned char* dx = g.dead_layer;
-    const unsigned char* dy = dx + g.nn[0];
-    const unsigned char* dz = dy + g.nn[1];
-    int x0 = -2, x1 = 2, y0 = -2, y1 = 2, z0 = -2, z1 = 2;
-    while (x0 <= 2 && (ia[0] + x0 < 0 || ia[0] + x0 > g.n[0] || dx[ia[0] + x0])) ++x0;
-    while (x1 >= x0 && (ia[0] + x1 < 0 || ia[0] + x1 > g.n[0] || dx[ia[0] + x1])) --x1;
-    while (y0 <= 2 && (ia[1] + y0 < 0 || ia[1] + y0 > g.n[1] || dy[ia[1] + y0])) ++y0;
-    while (y1 >= y0 && (ia[1] + y1 < 0 || ia[1] + y1 > g.n[1] || dy[ia[1] + y1])) --y1;
-    while (z0 <= 2 && (ia[2] + z0 < 0 || ia[2] + z0 > g.n[2] || dz[ia[2] + z0])) ++z0;
-    while (z1 >= z0 && (ia[2] + z1 < 0 || ia[2] + z1 > g.n[2] || dz[ia[2] + z1])) --z1;
-    rx = 3 * (x1 - x0 + 1);
-    ny = y1 - y0 + 1;
-    nv = x1 >= x0 && y1 >= y0 && z1 >= z0 ? rx * ny * (z1 - z0 + 1) : 0;
-    vbase = (z0 + 2) * 75 + (y0 + 2) * 15 + (x0 + 2) * 3;
-  }
-  // a patch whose node has every velocity component constrained owns only
-  // its pressure: its velocity rows are zero and only row d is summed
-  const bool wall = DIM == 3 && (mask[i] & 7) == 7;
-  const int tot = nv + P::NP;
-  int zi = 0, yi = 0, o = lane;  // loop index t = (zi ny + yi) rx + o while t < nv
-  if (nv > 0)
-    while (o >= rx) {
-      o -= rx;
-      if (++yi == ny) { yi = 0; ++zi; }
-    }
-  if (DIM == 3 && wall) {
-    for (int t = lane; t < tot; t += TPP) {
-      const int j = t < nv ? vbase + zi * 75 + yi * 15 + o : P::NU * DIM + (t - nv);
-      if (nv > 0) {
-        o += TPP;
-        while (o >= rx) {
-          o -= rx;
-          if (++yi == ny) { yi = 0; ++zi; }
-        }
-      }
-      y[ND - 1] += ldrow(cf + (size_t)j * ND + (ND - 1), shared_rows) * rp[soff[j]];
-    }
-  } else {
-#pragma unroll 4
-    for (int t = lane; t < tot; t += TPP) {
-      const int j = t < nv ? vbase + zi * 75 + yi * 15 + o : P::NU * DIM + (t - nv);
-      if (nv > 0) {
-        o += TPP;
-        while (o >= rx) {
-          o -= rx;
-          if (++yi == ny) { yi = 0; ++zi; }
-        }
-      }
-      double rv = rp[soff[j]];
-      if (ND == 4) {
-        const double2* c2 = reinterpret_cast<const double2*>(cf + (size_t)j * 4);
-        double2 a = ldrow(c2, shared_rows), b = ldrow(c2 + 1, shared_rows);
-        y[0] += a.x * rv; y[1] += a.y * rv; y[2] += b.x * rv; y[3] += b.y * rv;
-      } else {
-#pragma unroll
-        for (int k = 0; k < ND; ++k) y[k] += ldrow(cf + (size_t)j * ND + k, shared_rows) * rv;
-      }
-    }
-  }
-  if constexpr (TPP >= 4) {
-    // the lane whose group-lane bits below TPP/4 are zero writes component c
-    int c = 0;
-    const double yc = reduce_scatter4<TPP>(y, lane, &c);
-    if (valid && c < ND && (lane & (TPP / 4 - 1)) == 0) owned_update<ND>(i, c, mask, rp[c], yc, omega, x, nullptr);
-  } else {
-#pragma unroll
-    for (int k = 0; k < ND; ++k)
-#pragma unroll
-      for (int o = TPP / 2; o > 0; o >>= 1) y[k] += __shfl_xor_sync(0xffffffffu, y[k], o);
-    if (valid && lane < ND) owned_update<ND>(i, lane, mask, rp[lane], pick<ND>(y, lane), omega, x, nullptr);
-  }
+  const bool valid = gi < n;
+  const unsigned k = valid ? gi : n - 1;
+  apply_fp64_patch<DIM, TPP>(g, coef, mask, rpad, omega, x, prow, soff, LIST ? (unsigned)list[k] : k, valid);
 }
 
 // float32 / bfloat16 rows with float32 residual and float32 accumulation
@@ -3462,7 +3303,8 @@ cudaError_t launch_patch_rows_pair(const LevelGeom& g, const double* st, const u
 
 cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coef,
                                const unsigned char* mask, const double* rpad, const float* rpad32,
-                               double omega, double* x, const int* prow, cudaStream_t s) {
+                               double omega, double* x, const int* prow, cudaStream_t s, const int* list,
+                               long long nlist) {
   const long long threads32 = g.nnodes * 32;
   const unsigned blocks = (unsigned)((threads32 + 255) / 256);
   // 2D: 4 lanes per patch (see apply_tpp); 3D: a warp per patch
@@ -3470,15 +3312,19 @@ cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coe
   if (prec == FC_PREC_FP64) {
     const int t = apply64_tpp(g.dim);
     const unsigned bl = (unsigned)((g.nnodes * t + 255) / 256);
+    const unsigned nl = (unsigned)nlist;
     const double* c = (const double*)coef;
-    if (g.dim == 2) {
-      apply_fp64_kernel<2, 4><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow);
+    if (list) {
+      apply_fp64_kernel<3, 8, true>
+          <<<(unsigned)((nlist * 8 + 255) / 256), 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl);
+    } else if (g.dim == 2) {
+      apply_fp64_kernel<2, 4, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0);
     } else {
       switch (t) {
-        case 4: apply_fp64_kernel<3, 4><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow); break;
-        case 16: apply_fp64_kernel<3, 16><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow); break;
-        case 32: apply_fp64_kernel<3, 32><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow); break;
-        default: apply_fp64_kernel<3, 8><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow); break;
+        case 4: apply_fp64_kernel<3, 4, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0); break;
+        case 16: apply_fp64_kernel<3, 16, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0); break;
+        case 32: apply_fp64_kernel<3, 32, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0); break;
+        default: apply_fp64_kernel<3, 8, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0); break;
       }
     }
   } else if (prec == FC_PREC_FP32) {
