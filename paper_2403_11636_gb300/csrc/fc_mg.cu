@@ -502,8 +502,13 @@ __global__ void gemv_kernel(int n, const double* __restrict__ A, const double* _
 }
 
 // ---------------------------------------------------------------------------
-// deterministic reductions: a fixed grid of partial sums, then one block
-constexpr int kRedBlocks = 1024;
+// deterministic reductions: a grid of partial sums fixed by the length, then
+// one block.  Every block of a fused Gram-Schmidt step first adds up all the
+// partials of the step before, so their number is part of each launch's time:
+// 4 values a thread until 608 blocks (4 CTAs per SM) are there.  With 1024
+// blocks for any length a step took 12.6 us on 3,267 DoFs and 18 us on 1.1 M.
+constexpr int kRedBlocks = 608;
+inline int red_blocks(long long n) { return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + 1023) / 1024)); }
 
 __global__ void dot_partial_kernel(long long n, const double* __restrict__ a, const double* __restrict__ b,
                                    double* __restrict__ partial) {
@@ -851,8 +856,9 @@ cudaError_t launch_dense_gemv(int n, const double* A, const double* x, double* y
 
 cudaError_t launch_dot(long long n, const double* a, const double* b, double* partial, double* out,
                        cudaStream_t s) {
-  dot_partial_kernel<<<kRedBlocks, 256, 0, s>>>(n, a, b, partial);
-  sum_partial_kernel<<<1, 1024, 0, s>>>(kRedBlocks, partial, out);
+  const int nb = red_blocks(n);
+  dot_partial_kernel<<<nb, 256, 0, s>>>(n, a, b, partial);
+  sum_partial_kernel<<<1, nb <= 256 ? 256 : 1024, 0, s>>>(nb, partial, out);
   note_launches(2);
   return cudaGetLastError();
 }
@@ -860,8 +866,8 @@ cudaError_t launch_dot(long long n, const double* a, const double* b, double* pa
 cudaError_t launch_mgs_fused(long long n, double* w, const double* v_prev, const double* part_in,
                              double* h_out, const double* v_next, double* part_out, int finish,
                              double* v_out, double* hn_copy, cudaStream_t s) {
-  mgs_fused_kernel<<<kRedBlocks, 256, 0, s>>>(n, w, v_prev, part_in, h_out, v_next, part_out, finish, v_out,
-                                              hn_copy);
+  mgs_fused_kernel<<<red_blocks(n), 256, 0, s>>>(n, w, v_prev, part_in, h_out, v_next, part_out, finish, v_out,
+                                                 hn_copy);
   note_launches(1);
   return cudaGetLastError();
 }
