@@ -376,40 +376,62 @@ __global__ void q2_prolong_kernel(Q2Grid f, Q2Grid c, const unsigned char* __res
 }
 
 // restriction as a gather over the fine DoFs that interpolate from each
-// coarse DoF (the same weights as the prolongation, transposed)
+// coarse DoF (the same weights as the prolongation, transposed).  A thread per
+// velocity component of a coarse node (then one per vertex): the weights of
+// its at most 9 fine nodes per direction are found once, and of these at most
+// 5 are not zero (a node's function at its neighbours' quarter points).  With a
+// thread per node that formed all 729 products of weights, the two transfers of
+// a 16^3 cycle took 1.85 of its 5.7 ms.
 template <int DIM>
 __global__ void q2_restrict_kernel(Q2Grid f, Q2Grid c, const unsigned char* __restrict__ cmask,
                                    const double* __restrict__ rf, double* __restrict__ bc) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < c.nq) {
+  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool vel = id < c.nq * DIM;
+  const long long t = vel ? id / DIM : c.nq + (id - c.nq * DIM);
+  if (vel) {
+    const int cc = (int)(id - t * DIM);
     int J[3];
     q2_decode(c.nf, DIM, t, J);
-    double s[3] = {0.0, 0.0, 0.0};
+    double s = 0.0;
     if (!cmask[t]) {
       // fine Q2 nodes F with F / 4 in the coarse cells touching J: F in [2J - 4, 2J + 4]
-      int flo[3] = {0, 0, 0}, fhi[3] = {0, 0, 0};
+      double wk[3][5];
+      int Fk[3][5], nk[3] = {0, 0, 1};
+      wk[2][0] = 1.0;
+      Fk[2][0] = 0;
+#pragma unroll
       for (int k = 0; k < DIM; ++k) {
-        flo[k] = max(0, 2 * J[k] - 4);
-        fhi[k] = min(f.nf[k] - 1, 2 * J[k] + 4);
+        int m = 0;
+#pragma unroll
+        for (int d = -4; d <= 4; ++d) {
+          const int F = 2 * J[k] + d;
+          if (F < 0 || F >= f.nf[k]) continue;
+          int base;
+          double w[3];
+          q2_fine_w(F, c.nv1[k] - 1, &base, w);
+          const int l = J[k] - base;
+          const double wl = l == 0 ? w[0] : l == 1 ? w[1] : l == 2 ? w[2] : 0.0;
+          if (wl == 0.0 || m == 5) continue;
+#pragma unroll
+          for (int q = 0; q < 5; ++q)
+            if (q == m) { wk[k][q] = wl; Fk[k][q] = F; }
+          ++m;
+        }
+        nk[k] = m;
       }
-      for (int Fz = flo[2]; Fz <= fhi[2]; ++Fz)
-        for (int Fy = flo[1]; Fy <= fhi[1]; ++Fy)
-          for (int Fx = flo[0]; Fx <= fhi[0]; ++Fx) {
-            const int F[3] = {Fx, Fy, Fz};
-            double wt = 1.0;
-            for (int k = 0; k < DIM; ++k) {
-              int base;
-              double w[3];
-              q2_fine_w(F[k], c.nv1[k] - 1, &base, w);
-              const int l = J[k] - base;
-              wt = (l >= 0 && l <= 2) ? wt * w[l] : 0.0;
-            }
-            if (wt == 0.0) continue;
-            const long long fi = q2_index(f.nf, F);
-            for (int cc = 0; cc < DIM; ++cc) s[cc] = s[cc] + wt * rf[fi * DIM + cc];
-          }
+#pragma unroll
+      for (int z = 0; z < (DIM == 3 ? 5 : 1); ++z)
+#pragma unroll
+        for (int y = 0; y < 5; ++y) {
+          if (z >= nk[2] || y >= nk[1]) continue;
+          const double wzy = wk[1][y] * wk[2][z];
+          const long long row = f.nf[0] * (Fk[1][y] + (long long)f.nf[1] * Fk[2][z]);
+#pragma unroll
+          for (int x = 0; x < 5; ++x)
+            if (x < nk[0]) s = s + wk[0][x] * wzy * rf[(row + Fk[0][x]) * DIM + cc];
+        }
     }
-    for (int cc = 0; cc < DIM; ++cc) bc[t * DIM + cc] = s[cc];
+    bc[t * DIM + cc] = s;
   } else if (t < c.nq + c.np) {
     const long long u = t - c.nq;
     int U[3];
@@ -545,8 +567,8 @@ cudaError_t launch_q2_prolong_add(int dim, const Q2Grid& f, const Q2Grid& c, con
 
 cudaError_t launch_q2_restrict(int dim, const Q2Grid& f, const Q2Grid& c, const unsigned char* cmask,
                                const double* rf, double* bc, cudaStream_t s) {
-  if (dim == 2) q2_restrict_kernel<2><<<blocks_for(c.nq + c.np), 256, 0, s>>>(f, c, cmask, rf, bc);
-  else q2_restrict_kernel<3><<<blocks_for(c.nq + c.np), 256, 0, s>>>(f, c, cmask, rf, bc);
+  if (dim == 2) q2_restrict_kernel<2><<<blocks_for(c.nq * 2 + c.np), 256, 0, s>>>(f, c, cmask, rf, bc);
+  else q2_restrict_kernel<3><<<blocks_for(c.nq * 3 + c.np), 256, 0, s>>>(f, c, cmask, rf, bc);
   note_launches(1);
   return cudaGetLastError();
 }
