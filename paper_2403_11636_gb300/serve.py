@@ -201,12 +201,16 @@ class BatchServer:
     over the requests in flight (state None for a request that has just
     joined), new requests joining and converged ones (or ones past
     ``max_iters`` iterations) leaving between cycles; a request's result
-    holds ``final_fn(state)`` of its last cycle as its solution."""
+    holds ``final_fn(state)`` of its last cycle as its solution.  ``join_s``:
+    how long an idle live driver that has one request ready waits for a second
+    whose setup is running (two requests cost a cycle little more than one;
+    setups of 20 ms, as short as the gaps between requests, would otherwise
+    never meet in a batch)."""
 
     def __init__(self, setup_fn: Callable, round_fn: Callable, release_fn: Callable, footprint_fn: Callable,
                  budget_bytes: float, slots: int, max_batch: int = 64, make_stream: Callable = lambda: None,
                  clock: Callable = time.perf_counter, gather_s: float = 0.0, cycle_fn: Optional[Callable] = None,
-                 max_iters: int = 400, final_fn: Callable = lambda state: state):
+                 max_iters: int = 400, final_fn: Callable = lambda state: state, join_s: float = 0.0):
         if slots < 1 or max_batch < 1:
             raise ValueError("slots and max_batch must be >= 1")
         self.setup_fn = setup_fn
@@ -222,6 +226,7 @@ class BatchServer:
         self.make_stream = make_stream
         self.clock = clock
         self.gather_s = gather_s
+        self.join_s = join_s
 
     @classmethod
     def gpu(cls, budget_bytes: float = 150e9, slots: int = 8, prec: str = "fp32", dedup: int = 1,
@@ -286,7 +291,7 @@ class BatchServer:
 
         return cls(setup, solve_round, release, footprint, budget_bytes, slots, max_batch,
                    make_stream=lambda: torch.cuda.Stream(), gather_s=gather_s,
-                   cycle_fn=solve_cycle if live else None, final_fn=final)
+                   cycle_fn=solve_cycle if live else None, final_fn=final, join_s=0.03)
 
     def run(self, requests: List[Request]) -> List[BatchResult]:
         """Serve ``requests`` (arrival times relative to the call) to completion."""
@@ -365,6 +370,10 @@ class BatchServer:
                 with lock:
                     while not st["ready"] and not active and not (st["done_admitting"] and st["setting_up"] == 0):
                         lock.wait(timeout=0.05)
+                    deadline = self.clock() + self.join_s
+                    while (not active and st["setting_up"] > 0 and len(st["ready"]) == 1 and self.max_batch > 1
+                           and self.clock() < deadline):
+                        lock.wait(timeout=min(0.01, max(0.0, deadline - self.clock())))
                     room = self.max_batch - len(active)
                     joining = st["ready"][:room]
                     del st["ready"][: len(joining)]
