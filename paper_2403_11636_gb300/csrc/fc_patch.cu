@@ -894,7 +894,11 @@ __global__ void __launch_bounds__(256, 3)
 //   z_p = S~^{-1} h,   u_c(centre) = z_c(centre) - w_c . z_p,
 // and the owned DoFs take omega D (u, p) (the restricted update).  Patches
 // whose record is dense (index >= 0) are left to the dense apply over its
-// node list.
+// node list.  FP64 and the chain of the band solves bound it (930 warp
+// instructions per patch, a step of a solve twice as long as its product), so
+// as many CTAs as possible share an SM: S~ LU waits in registers and takes the
+// band's place, D z that of z: 36 KB, six CTAs (44 KB, five, and B' D z by one
+// warp while two waited: 2.88 ms per 33^3 sweep).
 __global__ void __launch_bounds__(96)
     band_factor_apply_kernel(LevelGeom g, const double* __restrict__ st, const double* __restrict__ fac,
                              const int* __restrict__ fpiv, const unsigned char* __restrict__ mask,
@@ -905,9 +909,9 @@ __global__ void __launch_bounds__(96)
   constexpr int NU = P::NU, NP = P::NP, ND = P::ND, SP = P::SP;
   constexpr int v0 = 62, p0 = 13;
   __shared__ __align__(16) double sL[NU * kBand];
-  __shared__ double sS[NP * NP];
-  __shared__ double sz[DIM * NU], szd[DIM * NU];
-  __shared__ double sh[NP];
+  __shared__ double sz[DIM * NU];
+  __shared__ double sh[DIM][NP];
+  double* sS = sL;  // S~ LU, once the band solves are done
   __shared__ int spiv[NP];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long i = blockIdx.x;
@@ -923,9 +927,12 @@ __global__ void __launch_bounds__(96)
     const double2* src = reinterpret_cast<const double2*>(rec);
     double2* dst = reinterpret_cast<double2*>(sL);
     for (int e = tid; e < NU * kBand / 2; e += 96) dst[e] = __ldcs(src + e);
-    for (int e = tid; e < NP * NP; e += 96) sS[e] = rec[NU * kBand + e];
     if (tid < NP) spiv[tid] = ip[tid];
   }
+  constexpr int NS = (NP * NP + 95) / 96;
+  double sreg[NS];
+#pragma unroll
+  for (int e = 0; e < NS; ++e) sreg[e] = tid + 96 * e < NP * NP ? __ldcs(rec + NU * kBand + tid + 96 * e) : 0.0;
   const unsigned nx = (unsigned)g.nn[0], ny = (unsigned)g.nn[1];
   const int ia[3] = {(int)((unsigned)i % nx), (int)(((unsigned)i / nx) % ny), (int)((unsigned)i / (nx * ny))};
   const long long pbase = pad_node(g, ia[0], ia[1], ia[2]);
@@ -941,7 +948,7 @@ __global__ void __launch_bounds__(96)
     sz[e] = act ? du[v] * rpad[pn * ND + c] : 0.0;
   }
   __syncthreads();
-  {  // z_c = K~^{-1} (D r)_c, one warp per component; szd = D z_c
+  {  // z_c = K~^{-1} (D r)_c, one warp per component; then D z_c in its place
     double* y = sz + warp * NU;
     band_forward(sL, y, NU, 0, lane);
     __syncwarp();
@@ -949,8 +956,33 @@ __global__ void __launch_bounds__(96)
     __syncwarp();
     band_backward(sL, y, NU, lane);
     __syncwarp();
-    for (int t = lane; t < NU; t += 32) szd[warp * NU + t] = du[t] * y[t];
+    for (int t = lane; t < NU; t += 32) y[t] *= du[t];
+    __syncwarp();
+    // -B_c' D z_c, lane q (the components side by side)
+    if (lane < NP) {
+      const int q = lane, c = warp;
+      int oq[3];
+      prs_off<DIM>(q, oq);
+      double acc = 0.0;
+#pragma unroll 3
+      for (int t = 0; t < 27; ++t) {
+        const int d[3] = {t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1};
+        const int ov[3] = {oq[0] + d[0], oq[1] + d[1], oq[2] + d[2]};
+        const int v = (ov[0] + 2) + 5 * (ov[1] + 2) + 25 * (ov[2] + 2);
+        const int b0 = ia[0] + ov[0], b1 = ia[1] + ov[1], b2 = ia[2] + ov[2];
+        if (b0 < 0 || b0 > g.n[0] || b1 < 0 || b1 > g.n[1] || b2 < 0 || b2 > g.n[2]) continue;
+        // (D z_c is zero at constrained nodes)
+        const long long bn = b0 + (long long)g.nn[0] * (b1 + (long long)g.nn[1] * b2);
+        const int dvp[3] = {-d[0], -d[1], -d[2]};  // q relative to v
+        acc = fma(-st[((long long)nb_index<DIM>(dvp) * SP + 1 + c) * g.nnodes + bn], y[v], acc);
+      }
+      sh[c][q] = acc;
+    }
   }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < NS; ++e)
+    if (tid + 96 * e < NP * NP) sS[tid + 96 * e] = sreg[e];
   __syncthreads();
   if (warp == 0) {
     // h = D r_p - sum_c B~_c' z_c = dp (r_p - sum_c B_c' D z_c), lane q
@@ -963,33 +995,21 @@ __global__ void __launch_bounds__(96)
       const bool qin = c0 >= 0 && c0 <= g.n[0] && c1 >= 0 && c1 <= g.n[1] && c2 >= 0 && c2 <= g.n[2];
       if (qin) {
         const long long pq = pbase + oq[0] + px * (oq[1] + py * oq[2]);
-        double acc = rpad[pq * ND + DIM];
-        for (int t = 0; t < 27; ++t) {
-          const int d[3] = {t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1};
-          const int ov[3] = {oq[0] + d[0], oq[1] + d[1], oq[2] + d[2]};
-          const int v = (ov[0] + 2) + 5 * (ov[1] + 2) + 25 * (ov[2] + 2);
-          const int b0 = ia[0] + ov[0], b1 = ia[1] + ov[1], b2 = ia[2] + ov[2];
-          if (b0 < 0 || b0 > g.n[0] || b1 < 0 || b1 > g.n[1] || b2 < 0 || b2 > g.n[2]) continue;
-          const long long bn = b0 + (long long)g.nn[0] * (b1 + (long long)g.nn[1] * b2);
-          if (mask[bn] & 1) continue;
-          const int dvp[3] = {-d[0], -d[1], -d[2]};  // q relative to v
-          const long long base = (long long)nb_index<DIM>(dvp) * SP;
-          for (int c = 0; c < DIM; ++c) acc = fma(-st[(base + 1 + c) * g.nnodes + bn], szd[c * NU + v], acc);
-        }
-        hv = dp[q] * acc;
+        hv = dp[q] * (((rpad[pq * ND + DIM] + sh[0][q]) + sh[1][q]) + sh[2][q]);
       }
-      sh[q] = hv;
     }
+    __syncwarp();
+    if (lane < NP) sh[0][lane] = hv;
     __syncwarp();
     // z_p = S~^{-1} h: row interchanges, then lane r carries z_p(r) through
     // the column steps of L (unit) and U (reciprocal diagonal stored)
     if (lane == 0)
       for (int k = 0; k < NP; ++k) {
         const int pk = spiv[k];
-        if (pk != k) { const double t0 = sh[k]; sh[k] = sh[pk]; sh[pk] = t0; }
+        if (pk != k) { const double t0 = sh[0][k]; sh[0][k] = sh[0][pk]; sh[0][pk] = t0; }
       }
     __syncwarp();
-    double z = lane < NP ? sh[lane] : 0.0;
+    double z = lane < NP ? sh[0][lane] : 0.0;
     for (int k = 0; k < NP - 1; ++k) {
       const double zk = __shfl_sync(0xffffffffu, z, k);
       if (lane > k && lane < NP) z = fma(-sS[lane * NP + k], zk, z);
@@ -1004,7 +1024,7 @@ __global__ void __launch_bounds__(96)
     for (int c = 0; c < DIM; ++c) {
       double pc = lane < NP ? wv[c * NP + lane] * z : 0.0;
       for (int o = 16; o > 0; o >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, o);
-      y[c] = du[v0] * (sz[c * NU + v0] - pc);
+      y[c] = sz[c * NU + v0] - du[v0] * pc;
     }
     y[DIM] = dp[p0] * __shfl_sync(0xffffffffu, z, p0);
     if (lane == 0) {
