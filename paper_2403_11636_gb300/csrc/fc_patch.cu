@@ -3197,15 +3197,20 @@ __global__ void __launch_bounds__(512)
   }
 }
 
-// 3D apply: a warp per vertex; lane l sums the 25 rows over the slots
-// l, l + 32, ... (coalesced row loads, residual gathers from the padded
-// copies), a reduce-scatter leaves row l's sum in lane l, and lanes 0..24
-// write the restricted update of the owned DoFs.
-__global__ void __launch_bounds__(256)
+// apply: five warps per vertex, five of the 25 owned rows each (y_k = sum_slots
+// rows[k][slot] r[slot]), the lanes striding over the slots; restricted update
+// as in 2D.  CTAs walk over the vertices, so the table of residual offsets is
+// built once.  FP64 bounds it (0.27 GFMA at 17^3 vertices, 432 us at the pipe's
+// rate).  A warp with all 25 rows of a vertex left 4,913 warps for 2,432 places
+// of the GPU, the last seven CTAs alone with a sixth of the time, and added up
+// 31 partial sums per lane for 1,750 products.
+constexpr int kQ2ApplyWarps = 5, kQ2ApplyCtas = 152 * 12;
+__global__ void __launch_bounds__(kQ2ApplyWarps * 32)
     q2_apply3_kernel(Q2Grid q, const double* __restrict__ coef, const unsigned char* __restrict__ mask,
                      const double* __restrict__ rpv, const double* __restrict__ rpp, double omega,
                      double* __restrict__ x) {
   using P = Q2P3;
+  constexpr int NR = P::NROW / kQ2ApplyWarps;
   __shared__ int soff[P::SP];
   const int PX = q.nf[0] + 8, PY = q.nf[1] + 8, PXP = q.nv1[0] + 2, PYP = q.nv1[1] + 2;
   for (int j = threadIdx.x; j < P::SP; j += blockDim.x) {
@@ -3220,46 +3225,44 @@ __global__ void __launch_bounds__(256)
     }
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const long long gv = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const bool valid = gv < q.np;
-  const long long v = valid ? gv : q.np - 1;
-  const int ax = (int)(v % q.nv1[0]), ay = (int)((v / q.nv1[0]) % q.nv1[1]),
-            az = (int)(v / ((long long)q.nv1[0] * q.nv1[1]));
-  const double* rv = rpv + (((long long)(2 * az + 4) * PY + (2 * ay + 4)) * PX + (2 * ax + 4)) * 3;
-  const double* rp = rpp + ((long long)(az + 1) * PYP + (ay + 1)) * PXP + (ax + 1);
-  const double* cf = coef + (size_t)v * P::NROW * P::SP;
-  double y[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (unsigned v = blockIdx.x; v < (unsigned)q.np; v += gridDim.x) {
+    const unsigned nx = (unsigned)q.nv1[0], ny = (unsigned)q.nv1[1];
+    const int ax = (int)(v % nx), ay = (int)((v / nx) % ny), az = (int)(v / (nx * ny));
+    const double* rv = rpv + (((long long)(2 * az + 4) * PY + (2 * ay + 4)) * PX + (2 * ax + 4)) * 3;
+    const double* rp = rpp + ((long long)(az + 1) * PYP + (ay + 1)) * PXP + (ax + 1);
+    const double* cf = coef + ((size_t)v * P::NROW + warp * NR) * P::SP;
+    double y[NR];
 #pragma unroll
-  for (int k = 0; k < 32; ++k) y[k] = 0.0;
-  for (int j = lane; j < P::SP; j += 32) {
-    const double r = j < P::NSV ? rv[soff[j]] : rp[soff[j]];
+    for (int k = 0; k < NR; ++k) y[k] = 0.0;
+#pragma unroll 4
+    for (int j = lane; j < P::SP; j += 32) {
+      const double r = j < P::NSV ? rv[soff[j]] : rp[soff[j]];
 #pragma unroll
-    for (int k = 0; k < P::NROW; ++k) y[k] += __ldcs(cf + (size_t)k * P::SP + j) * r;
-  }
-  // reduce-scatter over the 32 lanes: after the step of width w each lane
-  // keeps the half of its partial sums selected by bit w of its lane index
-#pragma unroll
-  for (int w = 16; w > 0; w >>= 1) {
-    const bool hi = lane & w;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const double send = hi ? y[i] : y[i + w];
-      const double keep = hi ? y[i + w] : y[i];
-      y[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+      for (int k = 0; k < NR; ++k) y[k] += __ldcs(cf + (size_t)k * P::SP + j) * r;
     }
-  }
-  if (!valid || lane >= P::NROW) return;
-  const double yk = y[0];
-  if (lane < 24) {
-    const int s = lane / 3, c = lane % 3;
-    const int I = 2 * ax + (s & 1), J = 2 * ay + ((s >> 1) & 1), K = 2 * az + (s >> 2);
-    if (I >= q.nf[0] || J >= q.nf[1] || K >= q.nf[2]) return;
-    const long long i = I + (long long)q.nf[0] * (J + (long long)q.nf[1] * K);
-    const double add = mask[i] ? rv[((s & 1) + PX * (((s >> 1) & 1) + PY * (s >> 2))) * 3 + c] : omega * yk;
-    x[i * 3 + c] += add;
-  } else {
-    x[q.nq * 3 + v] += omega * yk;
+    // rows 0-3 of the warp reduce-scattered, row 4 summed by all lanes
+    int row = 0;
+    double yk = reduce_scatter4<32>(y, lane, &row);
+    double y4 = y[4];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) y4 += __shfl_xor_sync(0xffffffffu, y4, o);
+    if ((lane & 7) != 0 && lane != 1) continue;
+    if (lane == 1) {
+      row = 4;
+      yk = y4;
+    }
+    const int k = warp * NR + row;
+    if (k < 24) {
+      const int s = k / 3, c = k % 3;
+      const int I = 2 * ax + (s & 1), J = 2 * ay + ((s >> 1) & 1), K = 2 * az + (s >> 2);
+      if (I >= q.nf[0] || J >= q.nf[1] || K >= q.nf[2]) continue;
+      const long long i = I + (long long)q.nf[0] * (J + (long long)q.nf[1] * K);
+      const double add = mask[i] ? rv[((s & 1) + PX * (((s >> 1) & 1) + PY * (s >> 2))) * 3 + c] : omega * yk;
+      x[i * 3 + c] += add;
+    } else {
+      x[q.nq * 3 + v] += omega * yk;
+    }
   }
 }
 
@@ -3503,8 +3506,8 @@ cudaError_t launch_q2_patch_rows(int dim, const Q2Grid& q, const double* A, cons
 cudaError_t launch_q2_apply(int dim, const Q2Grid& q, const double* coef, const unsigned char* mask, const double* rpv,
                             const double* rpp, double omega, double* x, cudaStream_t s) {
   if (dim == 3) {
-    const long long threads = q.np * 32;
-    q2_apply3_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(q, coef, mask, rpv, rpp, omega, x);
+    const unsigned ctas = (unsigned)std::min<long long>(q.np, kQ2ApplyCtas);
+    q2_apply3_kernel<<<ctas, kQ2ApplyWarps * 32, 0, s>>>(q, coef, mask, rpv, rpp, omega, x);
   } else {
     const long long threads = q.np * 8;
     q2_apply_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(q, coef, mask, rpv, rpp, omega, x);

@@ -243,24 +243,28 @@ __global__ void q2_rhs_kernel(LevelGeom g, Q2Grid q, const double* __restrict__ 
 // ---- residual r = b - L x (or L x when b is null); optional unpadded
 // output r and padded copies (velocity halo 4 nodes, pressure halo 1
 // vertex, zero halos) for the patch gathers
-template <int DIM>
+// TPP lanes per velocity node or vertex, each over every TPP-th neighbour: one
+// lane walks 152 blocks of a 3D node in turn, which on a 33^3 level left a
+// thread per node waiting for its loads (68 us a launch, 26 us of FP64).
+template <int DIM, int TPP>
 __global__ void __launch_bounds__(256)
     q2_residual_kernel(Q2Grid q, const double* __restrict__ A, const double* __restrict__ B,
                        const double* __restrict__ T, const unsigned char* __restrict__ mask,
                        const double* __restrict__ x, const double* __restrict__ b, double* __restrict__ r,
                        double* __restrict__ rpv, double* __restrict__ rpp) {
   using D = Q2D<DIM>;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x % TPP;
+  const long long gt = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPP;
+  const bool valid = gt < q.nq + q.np;  // groups past the last take part in the shuffles
+  const long long t = valid ? gt : q.nq + q.np - 1;
+  const bool vel = t < q.nq;
   const double* xp = x + q.nq * DIM;
-  if (t < q.nq) {
-    const long long i = t;
-    int I[3];
-    q2_decode(q.nf, DIM, i, I);
-    double acc[3] = {0.0, 0.0, 0.0};
-    if (mask[i]) {
-      for (int c = 0; c < DIM; ++c) acc[c] = x[i * DIM + c];
-    } else {
-      for (int o = 0; o < D::W5; ++o) {
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  int I[3];
+  if (vel) {
+    q2_decode(q.nf, DIM, t, I);
+    if (!mask[t]) {
+      for (int o = lane; o < D::W5; o += TPP) {
         const int J[3] = {I[0] + o % 5 - 2, I[1] + (o / 5) % 5 - 2, DIM == 3 ? I[2] + o / 25 - 2 : 0};
         bool in = true;
         for (int k = 0; k < DIM; ++k)
@@ -268,10 +272,11 @@ __global__ void __launch_bounds__(256)
         if (!in) continue;
         const long long j = q2_index(q.nf, J);
         if (mask[j]) continue;
-        const double a = A[(long long)o * q.nq + i];
+        const double a = A[(long long)o * q.nq + t];
+#pragma unroll
         for (int c = 0; c < DIM; ++c) acc[c] = acc[c] + a * x[j * DIM + c];
       }
-      for (int o = 0; o < D::W3; ++o) {
+      for (int o = lane; o < D::W3; o += TPP) {
         int V[3] = {0, 0, 0};
         bool in = true;
         const int off[3] = {o % 3, (o / 3) % 3, DIM == 3 ? o / 9 : 0};
@@ -281,40 +286,53 @@ __global__ void __launch_bounds__(256)
         }
         if (!in) continue;
         const double pv = xp[q2_index(q.nv1, V)];
-        for (int c = 0; c < DIM; ++c) acc[c] = acc[c] + B[((long long)o * DIM + c) * q.nq + i] * pv;
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) acc[c] = acc[c] + B[((long long)o * DIM + c) * q.nq + t] * pv;
       }
     }
-    long long pq = 0;
-    if (rpv) {
-      int P[3] = {I[0] + 4, I[1] + 4, DIM == 3 ? I[2] + 4 : 0};
-      pq = P[0] + (long long)(q.nf[0] + 8) * (P[1] + (long long)(q.nf[1] + 8) * P[2]);
-    }
-    for (int c = 0; c < DIM; ++c) {
-      const double v = b ? b[i * DIM + c] - acc[c] : acc[c];
-      if (r) r[i * DIM + c] = v;
-      if (rpv) rpv[pq * DIM + c] = v;
-    }
-  } else if (t < q.nq + q.np) {
+  } else {
     const long long v = t - q.nq;
-    int V[3];
-    q2_decode(q.nv1, DIM, v, V);
-    double acc = 0.0;
-    for (int o = 0; o < D::W5; ++o) {
-      const int J[3] = {2 * V[0] + o % 5 - 2, 2 * V[1] + (o / 5) % 5 - 2, DIM == 3 ? 2 * V[2] + o / 25 - 2 : 0};
+    q2_decode(q.nv1, DIM, v, I);
+    for (int o = lane; o < D::W5; o += TPP) {
+      const int J[3] = {2 * I[0] + o % 5 - 2, 2 * I[1] + (o / 5) % 5 - 2, DIM == 3 ? 2 * I[2] + o / 25 - 2 : 0};
       bool in = true;
       for (int k = 0; k < DIM; ++k)
         if (J[k] < 0 || J[k] >= q.nf[k]) in = false;
       if (!in) continue;
       const long long j = q2_index(q.nf, J);
       if (mask[j]) continue;
-      for (int c = 0; c < DIM; ++c) acc = acc + T[((long long)o * DIM + c) * q.np + v] * x[j * DIM + c];
+#pragma unroll
+      for (int c = 0; c < DIM; ++c) acc[0] = acc[0] + T[((long long)o * DIM + c) * q.np + v] * x[j * DIM + c];
     }
-    const double val = b ? b[q.nq * DIM + v] - acc : acc;
-    if (r) r[q.nq * DIM + v] = val;
-    if (rpp) {
-      const int P[3] = {V[0] + 1, V[1] + 1, DIM == 3 ? V[2] + 1 : 0};
-      rpp[P[0] + (long long)(q.nv1[0] + 2) * (P[1] + (long long)(q.nv1[1] + 2) * P[2])] = val;
+  }
+  // component c of a node (a vertex: c = 0) by the lane that holds its sum
+  auto store = [&](int c, double sum) {
+    if (vel) {
+      const double y = mask[t] ? x[t * DIM + c] : sum;
+      const double val = b ? b[t * DIM + c] - y : y;
+      if (r) r[t * DIM + c] = val;
+      if (rpv) {
+        const int P[3] = {I[0] + 4, I[1] + 4, DIM == 3 ? I[2] + 4 : 0};
+        rpv[(P[0] + (long long)(q.nf[0] + 8) * (P[1] + (long long)(q.nf[1] + 8) * P[2])) * DIM + c] = val;
+      }
+    } else if (c == 0) {
+      const long long v = t - q.nq;
+      const double val = b ? b[q.nq * DIM + v] - sum : sum;
+      if (r) r[q.nq * DIM + v] = val;
+      if (rpp) {
+        const int P[3] = {I[0] + 1, I[1] + 1, DIM == 3 ? I[2] + 1 : 0};
+        rpp[P[0] + (long long)(q.nv1[0] + 2) * (P[1] + (long long)(q.nv1[1] + 2) * P[2])] = val;
+      }
     }
+  };
+  if constexpr (TPP == 1) {
+    if (!valid) return;
+#pragma unroll
+    for (int c = 0; c < DIM; ++c) store(c, acc[c]);
+  } else {
+    int c = 0;
+    const double sum = reduce_scatter4<TPP>(acc, lane, &c);
+    if (valid && c < DIM && (lane & (TPP / 4 - 1)) == 0) store(c, sum);
   }
 }
 
@@ -551,8 +569,14 @@ cudaError_t launch_q2_assemble(const LevelGeom& g, const Q2Grid& q, const double
 cudaError_t launch_q2_residual(int dim, const Q2Grid& q, const double* A, const double* B, const double* T,
                                const unsigned char* mask, const double* x, const double* b, double* r, double* rpv,
                                double* rpp, cudaStream_t s) {
-  if (dim == 2) q2_residual_kernel<2><<<blocks_for(q.nq + q.np), 256, 0, s>>>(q, A, B, T, mask, x, b, r, rpv, rpp);
-  else q2_residual_kernel<3><<<blocks_for(q.nq + q.np), 256, 0, s>>>(q, A, B, T, mask, x, b, r, rpv, rpp);
+  const long long n = q.nq + q.np;
+  if (dim == 3) {
+    q2_residual_kernel<3, 8><<<blocks_for(n * 8), 256, 0, s>>>(q, A, B, T, mask, x, b, r, rpv, rpp);
+  } else if (n < 152 * 256) {
+    q2_residual_kernel<2, 4><<<blocks_for(n * 4), 256, 0, s>>>(q, A, B, T, mask, x, b, r, rpv, rpp);
+  } else {
+    q2_residual_kernel<2, 1><<<blocks_for(n), 256, 0, s>>>(q, A, B, T, mask, x, b, r, rpv, rpp);
+  }
   note_launches(1);
   return cudaGetLastError();
 }
