@@ -310,7 +310,9 @@ bool f32_path(fc_handle h) {
 // Float-pair smoothing: x and (unless already current) b are split into
 // pairs once, then every sweep is a pair residual and a pair apply that
 // keeps the pair copy of x current.
-fc_status smooth_level_pairs(fc_handle h, int li, double* x, const double* b, int nsweeps, bool b_current) {
+// zero: x is zero, the first residual is b.
+fc_status smooth_level_pairs(fc_handle h, int li, double* x, const double* b, int nsweeps, bool b_current,
+                             bool zero = false) {
   Level& L = h->lev[li];
   if (nsweeps <= 0) return FC_OK;
   CK(launch_split_x_padded(L.g, x, L.xp2, h->stream));
@@ -318,7 +320,8 @@ fc_status smooth_level_pairs(fc_handle h, int li, double* x, const double* b, in
   for (int s = 0; s < nsweeps; ++s) {
     {
       ProfScope ps(h, 1, 0.0);
-      CK(launch_residual_df2(L.g, L.st2, L.mask, L.xp2, L.bp2, (float2*)L.rpad32, nullptr, h->stream));
+      if (zero && s == 0) CK(launch_split_x_padded(L.g, b, (float2*)L.rpad32, h->stream));
+      else CK(launch_residual_df2(L.g, L.st2, L.mask, L.xp2, L.bp2, (float2*)L.rpad32, nullptr, h->stream));
     }
     ProfScope ps(h, 0, level_apply_bytes(h, li));
     ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, level_apply_bytes(h, li));
@@ -335,18 +338,20 @@ cudaError_t level_residual(fc_handle h, int li, const double* x, const double* b
 cudaError_t level_restrict(fc_handle h, int li, const double* rf, double* bc);
 cudaError_t level_prolong_add(fc_handle h, int li, const double* ec, double* xf);
 
-fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nsweeps) {
+// zero: x is zero, so the residual of the first sweep is b itself
+fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nsweeps, bool zero = false) {
   Level& L = h->lev[li];
-  if (pair_path(h)) return smooth_level_pairs(h, li, x, b, nsweeps, false);
+  if (pair_path(h)) return smooth_level_pairs(h, li, x, b, nsweeps, false, zero);
   if (amr_path(h)) {
     for (int s = 0; s < nsweeps; ++s) {
-      {
+      const bool from_b = zero && s == 0;
+      if (!from_b) {
         ProfScope ps(h, 1, 0.0);
         CK(launch_amr_residual(L.amr, x, b, L.r, h->stream));
       }
       ProfScope ps(h, 0, (double)L.coef_bytes);
       ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, (double)L.coef_bytes);
-      CK(launch_amr_apply(L.amr, L.r, h->opt.omega, x, h->stream));
+      CK(launch_amr_apply(L.amr, from_b ? b : L.r, h->opt.omega, x, h->stream));
     }
     return FC_OK;
   }
@@ -354,8 +359,8 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
     for (int s = 0; s < nsweeps; ++s) {
       {
         ProfScope ps(h, 1, 0.0);
-        CK(launch_q2_residual(h->dim, L.q2, L.q2A, L.q2B, L.q2T, L.q2mask, x, b, nullptr, L.q2rpv, L.q2rpp,
-                              h->stream));
+        CK(launch_q2_residual(h->dim, L.q2, L.q2A, L.q2B, L.q2T, L.q2mask, zero && s == 0 ? nullptr : x, b, nullptr,
+                              L.q2rpv, L.q2rpp, h->stream));
       }
       ProfScope ps(h, 0, (double)L.coef_bytes);
       ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, (double)L.coef_bytes);
@@ -365,8 +370,13 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
     return FC_OK;
   }
   for (int s = 0; s < nsweeps; ++s) {
-    fc_status st = smoother_residual(h, li, x, b);
-    if (st != FC_OK) return st;
+    if (zero && s == 0 && (h->opt.cache != FC_CACHE_INVERSE || h->opt.prec == FC_PREC_FP64)) {
+      ProfScope ps(h, 1, 0.0);
+      CK(launch_pad_rhs(L.g, b, L.rpad, h->stream));
+    } else {
+      const fc_status st = smoother_residual(h, li, x, b);
+      if (st != FC_OK) return st;
+    }
     if (h->opt.cache == FC_CACHE_INVERSE) {
       ProfScope ps(h, 0, level_apply_bytes(h, li));
       ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, level_apply_bytes(h, li));
@@ -383,7 +393,7 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
   return FC_OK;
 }
 
-fc_status vcycle_level(fc_handle h, int li, double* x, const double* b);
+fc_status vcycle_level(fc_handle h, int li, double* x, const double* b, bool zero);
 
 // Class products of a level on the tensor cores (fc_digits.cu): the plan is
 // kept where it pays.
@@ -441,6 +451,14 @@ fc_status coarse_part(fc_handle h) {
   Level& C = h->lev[li - 1];
   if (!h->coarse_graph) {
     cudaGraph_t graph = nullptr;
+    // a legacy or per-thread default stream cannot be captured: the launches
+    // are recorded on a stream of their own, and the graph runs on the
+    // handle's.  (Profiled launches record events: not while capturing.)
+    cudaStream_t const run = h->stream;
+    if (run == nullptr || run == cudaStreamLegacy || run == cudaStreamPerThread) {
+      if (!h->cap) CK(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
+      h->stream = h->cap;
+    }
     h->capturing = true;
     fc::g_capturing = true;
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
@@ -449,11 +467,12 @@ fc_status coarse_part(fc_handle h) {
       if (level_restrict(h, li, L.r, C.b) != cudaSuccess ||
           cudaMemsetAsync(C.x, 0, sizeof(double) * C.g.ndof, h->stream) != cudaSuccess)
         st = FC_ERR_CUDA;
-      if (st == FC_OK) st = vcycle_level(h, li - 1, C.x, C.b);
+      if (st == FC_OK) st = vcycle_level(h, li - 1, C.x, C.b, true);
       e = cudaStreamEndCapture(h->stream, &graph);
     }
     h->capturing = false;
     fc::g_capturing = false;
+    h->stream = run;
     if (e != cudaSuccess || st != FC_OK) {
       if (graph) cudaGraphDestroy(graph);
       return e != cudaSuccess ? cuda_fail(h, e, "V-cycle graph capture") : st;
@@ -480,7 +499,8 @@ fc_status coarse_part(fc_handle h) {
   return FC_OK;
 }
 
-fc_status vcycle_level(fc_handle h, int li, double* x, const double* b) {
+// zero: x is zero on entry
+fc_status vcycle_level(fc_handle h, int li, double* x, const double* b, bool zero) {
   Level& L = h->lev[li];
   if (li == 0) {
     CK(launch_dense_gemv(h->coarse_n, h->coarse_inv, b, x, h->stream));
@@ -493,25 +513,24 @@ fc_status vcycle_level(fc_handle h, int li, double* x, const double* b) {
     // pairs, so the residual for the restriction is a pair residual too
     CK(launch_split_pairs(L.g.ndof, b, L.bp2, h->stream));
     if (h->opt.nu_pre > 0) {
-      st = smooth_level_pairs(h, li, x, b, h->opt.nu_pre, true);
+      st = smooth_level_pairs(h, li, x, b, h->opt.nu_pre, true, zero);
       if (st != FC_OK) return st;
     } else {
       CK(launch_split_x_padded(L.g, x, L.xp2, h->stream));
     }
     CK(launch_residual_df2(L.g, L.st2, L.mask, L.xp2, L.bp2, nullptr, L.r, h->stream));
   } else {
-    st = smooth_level(h, li, x, b, h->opt.nu_pre);
+    st = smooth_level(h, li, x, b, h->opt.nu_pre, zero);
     if (st != FC_OK) return st;
     CK(level_residual(h, li, x, b, L.r));
   }
-  if (li == h->nlev - 1 && h->stream != nullptr && h->stream != cudaStreamLegacy &&
-      h->stream != cudaStreamPerThread) {
-    // (the legacy default stream cannot be captured; it runs the launches directly)
+  const bool legacy = h->stream == nullptr || h->stream == cudaStreamLegacy || h->stream == cudaStreamPerThread;
+  if (li == h->nlev - 1 && !(legacy && h->prof.on)) {  // (the profiler times every launch on a default stream)
     st = coarse_part(h);
   } else {
     CK(level_restrict(h, li, L.r, C.b));
     CK(cudaMemsetAsync(C.x, 0, sizeof(double) * C.g.ndof, h->stream));
-    st = vcycle_level(h, li - 1, C.x, C.b);
+    st = vcycle_level(h, li - 1, C.x, C.b, true);
   }
   if (st != FC_OK) return st;
   CK(level_prolong_add(h, li, C.x, x));
@@ -1500,7 +1519,7 @@ fc_status fc_vcycle(fc_handle h, double* x, const double* b) {
   if (!x || !b) return fail(h, FC_ERR_INVALID, "null vector");
   ProfScope ps(h, 2, 0.0);
   if (f32_path(h)) return handle_vcycle_f32(h, x, b, false);
-  return vcycle_level(h, h->nlev - 1, x, b);
+  return vcycle_level(h, h->nlev - 1, x, b, false);
 }
 
 fc_status fc_solve(fc_handle h, const double* b, double* x, double rtol, int maxit, int* iters,
@@ -1549,7 +1568,7 @@ fc_status fc_solve(fc_handle h, const double* b, double* x, double rtol, int max
       CK(cudaMemsetAsync(Zj, 0, sizeof(double) * n, s));
       {
         ProfScope ps(h, 2, 0.0);
-        st = f32_path(h) ? handle_vcycle_f32(h, Zj, Vj, true) : vcycle_level(h, h->nlev - 1, Zj, Vj);
+        st = f32_path(h) ? handle_vcycle_f32(h, Zj, Vj, true) : vcycle_level(h, h->nlev - 1, Zj, Vj, true);
         if (st != FC_OK) return st;
       }
       its++;
@@ -1557,19 +1576,23 @@ fc_status fc_solve(fc_handle h, const double* b, double* x, double rtol, int max
       // modified Gram-Schmidt, one fused kernel per step: step i finishes
       // h_{i-1,j} from the block partials, subtracts it and starts the dot
       // with v_i; the last two steps give the norm and v_{j+1}
-      double* pa = h->red;
-      double* pb = h->red + 1024;
-      CK(launch_mgs_fused(n, h->w, nullptr, nullptr, nullptr, h->V, pa, 0, nullptr, nullptr, s));
-      for (int i = 1; i <= j + 1; ++i) {
-        const double* vnext = i <= j ? h->V + (long long)i * n : nullptr;
-        CK(launch_mgs_fused(n, h->w, h->V + (long long)(i - 1) * n, pa, H + (long long)(i - 1) * m + j, vnext,
-                            pb, 0, nullptr, nullptr, s));
-        std::swap(pa, pb);
+      if (mgs_fits_cta(n)) {
+        CK(launch_mgs_small(n, h->w, h->V, H, m, j, bn, s));
+      } else {
+        double* pa = h->red;
+        double* pb = h->red + 1024;
+        CK(launch_mgs_fused(n, h->w, nullptr, nullptr, nullptr, h->V, pa, 0, nullptr, nullptr, s));
+        for (int i = 1; i <= j + 1; ++i) {
+          const double* vnext = i <= j ? h->V + (long long)i * n : nullptr;
+          CK(launch_mgs_fused(n, h->w, h->V + (long long)(i - 1) * n, pa, H + (long long)(i - 1) * m + j, vnext,
+                              pb, 0, nullptr, nullptr, s));
+          std::swap(pa, pb);
+        }
+        double* hn = H + (long long)(j + 1) * m + j;
+        CK(launch_mgs_fused(n, h->w, nullptr, pa, hn, nullptr, nullptr, 1, h->V + (long long)(j + 1) * n, sc + 2,
+                            s));
+        CK(launch_givens(H, m, j, bn, s));
       }
-      double* hn = H + (long long)(j + 1) * m + j;
-      CK(launch_mgs_fused(n, h->w, nullptr, pa, hn, nullptr, nullptr, 1, h->V + (long long)(j + 1) * n, sc + 2,
-                          s));
-      CK(launch_givens(H, m, j, bn, s));
       CK(cudaMemcpyAsync(h->host_small, sc, sizeof(double) * 3, cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
       double est = h->host_small[0], hnv = h->host_small[2];
@@ -1605,7 +1628,7 @@ fc_status fc_gmg_solve(fc_handle h, const double* b, double* x, double reduction
   while (it < maxit && rn > reduction * r0) {
     {
       ProfScope ps(h, 2, 0.0);
-      st = f32_path(h) ? handle_vcycle_f32(h, x, b, false) : vcycle_level(h, h->nlev - 1, x, b);
+      st = f32_path(h) ? handle_vcycle_f32(h, x, b, false) : vcycle_level(h, h->nlev - 1, x, b, false);
       if (st != FC_OK) return st;
     }
     CK(level_residual(h, h->nlev - 1, x, b, h->w));
@@ -1797,6 +1820,7 @@ fc_status fc_destroy(fc_handle h) {
     dfree(h, L.amr.rrp); dfree(h, L.amr.rcl); dfree(h, L.amr.rvl);
   }
   if (h->coarse_graph) cudaGraphExecDestroy(h->coarse_graph);
+  if (h->cap) cudaStreamDestroy(h->cap);
   dfree(h, h->d_shapes); dfree(h, h->d_err); dfree(h, h->coarse_inv);
   dfree(h, h->V); dfree(h, h->Z); dfree(h, h->w); dfree(h, h->red); dfree(h, h->small);
   dfree(h, h->bh); dfree(h, h->xh);

@@ -294,6 +294,7 @@ struct fc_handle_s {
   fc::Shape* d_shapes = nullptr;
   int nshape = 0;
   unsigned* d_err = nullptr;
+  cudaStream_t cap = nullptr;  // only captures (coarse_part); nothing runs on it
   // coarse solve: dense inverse of the coarsest operator
   double* coarse_inv = nullptr;
   int coarse_n = 0;
@@ -422,6 +423,8 @@ cudaError_t launch_rhs(const LevelGeom& g, const double* eF, const double* st,
 cudaError_t launch_residual(const LevelGeom& g, const double* st, const unsigned char* mask,
                             const double* x, const double* b, double* r, double* rpad,
                             cudaStream_t s);
+// rpad <- b (the smoother residual of x = 0)
+cudaError_t launch_pad_rhs(const LevelGeom& g, const double* b, double* rpad, cudaStream_t s);
 cudaError_t launch_residual_df(const LevelGeom& g, const double* st, const unsigned char* mask,
                                const double* x, const double* b, float* rpad2, cudaStream_t s);
 cudaError_t launch_residual_f32(const LevelGeom& g, const double* st, const unsigned char* mask,
@@ -571,6 +574,11 @@ cudaError_t launch_mgs_step(long long n, double* w, const double* vi, const doub
 cudaError_t launch_mgs_fused(long long n, double* w, const double* v_prev, const double* part_in,
                              double* h_out, const double* v_next, double* part_out, int finish,
                              double* v_out, double* hn_copy, cudaStream_t s);
+// one Arnoldi step's orthogonalisation and rotations in one launch, for vectors
+// that mgs_fits_cta: w is left as it was, V_{j+1} and column j of H are written
+bool mgs_fits_cta(long long n);
+cudaError_t launch_mgs_small(long long n, const double* w, double* V, double* small, int m, int j, double bnorm,
+                             cudaStream_t s);
 cudaError_t launch_givens(double* small, int m, int j, double bnorm, cudaStream_t s);
 cudaError_t launch_update_x(long long n, int k, int m, const double* small, const double* Z,
                             double* x, cudaStream_t s);

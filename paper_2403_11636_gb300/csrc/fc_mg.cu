@@ -271,6 +271,17 @@ __global__ void merge_x_padded_kernel(LevelGeom g, const float2* __restrict__ xp
   }
 }
 
+// padded copy of a level's right-hand side: the residual of x = 0
+template <int ND>
+__global__ void pad_rhs_kernel(LevelGeom g, const double* __restrict__ b, double* __restrict__ rpad) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= g.ndof) return;
+  const unsigned node = (unsigned)(t / ND);
+  int ia[3];
+  decode_node<ND - 1>(g, node, ia);
+  rpad[pad_node(g, ia[0], ia[1], ia[2]) * ND + (t - (long long)node * ND)] = b[t];
+}
+
 __global__ void split_pairs_kernel(long long n, const double* __restrict__ in, float2* __restrict__ out) {
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     double v = in[t];
@@ -629,7 +640,7 @@ __global__ void mgs_step_kernel(long long n, double* __restrict__ w, const doubl
 // Small FGMRES state (device, one thread):
 //   H[(m+1) x m] row-major at small[0], cs[m], sn[m], g[m+1], y[m],
 //   scalars at the end: [est, hn, beta, ...]
-__global__ void givens_kernel(double* small, int m, int j, double bnorm) {
+__device__ __forceinline__ void givens_step(double* small, int m, int j, double bnorm) {
   double* H = small;
   double* cs = H + (m + 1) * m;
   double* sn = cs + m;
@@ -650,6 +661,70 @@ __global__ void givens_kernel(double* small, int m, int j, double bnorm) {
   g[j + 1] = -sn[j] * g[j];
   g[j] = cs[j] * g[j];
   sc[0] = fabs(g[j + 1]) / bnorm;
+}
+__global__ void givens_kernel(double* small, int m, int j, double bnorm) { givens_step(small, m, j, bnorm); }
+
+// The whole orthogonalisation of a short vector (at most kMgsSmall values, held
+// in the registers of one CTA): modified Gram-Schmidt against v_0 .. v_j, the
+// norm, v_{j+1}, and the rotations of givens_kernel.  On 3,267 DoFs a step of
+// the split form is 4.6 us and its launch as long again, j + 3 of them.
+constexpr int kMgsSmall = 8192, kMgsPer = kMgsSmall / 1024;
+
+__device__ __forceinline__ double cta_sum(double s, double* sm) {
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  __syncthreads();  // the sums of the call before are read
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double t = sm[threadIdx.x & 31];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+__global__ void __launch_bounds__(1024)
+    mgs_small_kernel(int n, const double* __restrict__ w, double* __restrict__ V, double* __restrict__ small, int m,
+                     int j, double bnorm) {
+  __shared__ double sm[32];
+  double* H = small;
+  double* sc = H + (long long)(m + 1) * m + 2 * m + (m + 1) + m;
+  double r[kMgsPer];
+#pragma unroll
+  for (int k = 0; k < kMgsPer; ++k) {
+    const int e = k * 1024 + threadIdx.x;
+    r[k] = e < n ? w[e] : 0.0;
+  }
+  for (int i = 0; i <= j; ++i) {
+    const double* v = V + (long long)i * n;
+    double vv[kMgsPer], s = 0.0;
+#pragma unroll
+    for (int k = 0; k < kMgsPer; ++k) {
+      const int e = k * 1024 + threadIdx.x;
+      vv[k] = e < n ? v[e] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kMgsPer; ++k)
+      if (k * 1024 < n) s = fma(r[k], vv[k], s);
+    const double h = cta_sum(s, sm);
+#pragma unroll
+    for (int k = 0; k < kMgsPer; ++k)
+      if (k * 1024 < n) r[k] = fma(-h, vv[k], r[k]);
+    if (threadIdx.x == 0) H[i * m + j] = h;
+  }
+  double s = 0.0;
+#pragma unroll
+  for (int k = 0; k < kMgsPer; ++k)
+    if (k * 1024 < n) s = fma(r[k], r[k], s);
+  const double hn = sqrt(cta_sum(s, sm));
+  const double f = hn != 0.0 ? 1.0 / hn : 0.0;
+#pragma unroll
+  for (int k = 0; k < kMgsPer; ++k) {
+    const int e = k * 1024 + threadIdx.x;
+    if (e < n) V[(long long)(j + 1) * n + e] = r[k] * f;
+  }
+  if (threadIdx.x == 0) {
+    H[(j + 1) * m + j] = hn;
+    sc[2] = hn;
+    givens_step(small, m, j, bnorm);
+  }
 }
 
 // y = H^{-1} g (k x k upper triangular), then x += sum_i y_i Z_i
@@ -725,6 +800,14 @@ cudaError_t launch_residual_f32(const LevelGeom& g, const double* st, const unsi
   unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
   if (g.dim == 2) residual_kernel<2, 2, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
   else residual_kernel<3, 2, 1><<<blocks, 256, 0, s>>>(g, st, mask, x, b, nullptr, nullptr, rpad);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pad_rhs(const LevelGeom& g, const double* b, double* rpad, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((g.ndof + 255) / 256);
+  if (g.dim == 2) pad_rhs_kernel<3><<<blocks, 256, 0, s>>>(g, b, rpad);
+  else pad_rhs_kernel<4><<<blocks, 256, 0, s>>>(g, b, rpad);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -868,6 +951,15 @@ cudaError_t launch_mgs_fused(long long n, double* w, const double* v_prev, const
                              double* v_out, double* hn_copy, cudaStream_t s) {
   mgs_fused_kernel<<<red_blocks(n), 256, 0, s>>>(n, w, v_prev, part_in, h_out, v_next, part_out, finish, v_out,
                                                  hn_copy);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+bool mgs_fits_cta(long long n) { return n <= kMgsSmall; }
+
+cudaError_t launch_mgs_small(long long n, const double* w, double* V, double* small, int m, int j, double bnorm,
+                             cudaStream_t s) {
+  mgs_small_kernel<<<1, 1024, 0, s>>>((int)n, w, V, small, m, j, bnorm);
   note_launches(1);
   return cudaGetLastError();
 }

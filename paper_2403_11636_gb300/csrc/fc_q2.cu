@@ -243,6 +243,7 @@ __global__ void q2_rhs_kernel(LevelGeom g, Q2Grid q, const double* __restrict__ 
 // ---- residual r = b - L x (or L x when b is null); optional unpadded
 // output r and padded copies (velocity halo 4 nodes, pressure halo 1
 // vertex, zero halos) for the patch gathers
+// x null: the residual of x = 0.
 // TPP lanes per velocity node or vertex, each over every TPP-th neighbour: one
 // lane walks 152 blocks of a 3D node in turn, which on a 33^3 level left a
 // thread per node waiting for its loads (68 us a launch, 26 us of FP64).
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256)
   int I[3];
   if (vel) {
     q2_decode(q.nf, DIM, t, I);
-    if (!mask[t]) {
+    if (x && !mask[t]) {
       for (int o = lane; o < D::W5; o += TPP) {
         const int J[3] = {I[0] + o % 5 - 2, I[1] + (o / 5) % 5 - 2, DIM == 3 ? I[2] + o / 25 - 2 : 0};
         bool in = true;
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(256)
   } else {
     const long long v = t - q.nq;
     q2_decode(q.nv1, DIM, v, I);
-    for (int o = lane; o < D::W5; o += TPP) {
+    for (int o = x ? lane : D::W5; o < D::W5; o += TPP) {
       const int J[3] = {2 * I[0] + o % 5 - 2, 2 * I[1] + (o / 5) % 5 - 2, DIM == 3 ? 2 * I[2] + o / 25 - 2 : 0};
       bool in = true;
       for (int k = 0; k < DIM; ++k)
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(256)
   // component c of a node (a vertex: c = 0) by the lane that holds its sum
   auto store = [&](int c, double sum) {
     if (vel) {
-      const double y = mask[t] ? x[t * DIM + c] : sum;
+      const double y = x && mask[t] ? x[t * DIM + c] : sum;
       const double val = b ? b[t * DIM + c] - y : y;
       if (r) r[t * DIM + c] = val;
       if (rpv) {
