@@ -217,6 +217,11 @@ struct RowLoad<1, ND> {
       for (int k = 0; k < ND; ++k) v[k] = ldr(p + k, c);
     }
   }
+  // ND == 4, shared memory
+  static __device__ __forceinline__ void load_shared(const float* p, float* v) {
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[ND - 1] = a.w;
+  }
 };
 template <int ND>
 struct RowLoad<2, ND> {
@@ -232,6 +237,11 @@ struct RowLoad<2, ND> {
 #pragma unroll
       for (int k = 0; k < ND; ++k) v[k] = __uint_as_float((unsigned)ldr(q + k, c) << 16);
     }
+  }
+  static __device__ __forceinline__ void load_shared(const __nv_bfloat16* p, float* v) {
+    const uint2 a = *reinterpret_cast<const uint2*>(p);
+    v[0] = __uint_as_float(a.x << 16); v[1] = __uint_as_float(a.x & 0xffff0000u);
+    v[2] = __uint_as_float(a.y << 16); v[ND - 1] = __uint_as_float(a.y & 0xffff0000u);
   }
 };
 
@@ -610,46 +620,137 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// One 2D patch's product by one thread, in the order of the TPP-lane sum: a
+// leaf (S == TPP) is lane LANE's, the slots LANE, LANE + TPP, ..., then the
+// lanes are added pairwise (l with l + TPP/2 first).  Depth first, so no more
+// than log2(TPP) + 1 partial rows are live.  A row's fourth float is the bits
+// of its slot's offset.
+template <int TPP, int S, int LANE>
+__device__ __forceinline__ void class_tree2(const float4* rows, const float* rp, float* y) {
+  constexpr int NSLOT = 59;
+  if constexpr (S == TPP) {
+    y[0] = y[1] = y[2] = 0.0f;
+#pragma unroll
+    for (int j = LANE; j < NSLOT; j += TPP) {
+      const float4 cv = rows[j];
+      const float rv = rp[__float_as_int(cv.w)];
+      y[0] = fmaf(cv.x, rv, y[0]);
+      y[1] = fmaf(cv.y, rv, y[1]);
+      y[2] = fmaf(cv.z, rv, y[2]);
+    }
+  } else {
+    float b[3];
+    class_tree2<TPP, 2 * S, LANE>(rows, rp, y);
+    class_tree2<TPP, 2 * S, LANE + S>(rows, rp, b);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) y[t] += b[t];
+  }
+}
+
+// Parts of a chunk in the float32 applies, for levels with too few chunks to
+// fill the SMs evenly: with whole chunks a 33^3 level ran 0.127 ms and a 17^3
+// level as long (every group had the same 8 patches in sequence), with parts
+// 0.047 and 0.009 ms (3D, float32 rows).  In 2D a part costs its own split
+// into class and other patches: 1216 and more items were slower on 48
+// problems of 64^2 to 111^2 (0.031 against 0.028 ms on their second level).
+template <int DIM>
+__host__ __device__ constexpr int apply_parts(int nch, int ngrp) {
+  int parts = kChunk > 32 * ngrp ? kChunk / (32 * ngrp) : 1;  // 32 patches a group at most
+  while (2 * parts * ngrp <= kChunk && (long long)nch * parts < (DIM == 3 ? 2432 : 608)) parts *= 2;
+  return parts;
+}
+
 // d += omega L_i^{-1} r on the owned DoFs (PT 1: float32 rows, 2: bfloat16).
-// The 2D loop is bound by the latency of its loads (rows from the cache for
-// the shared class blocks, residual gathers): three 512-thread CTAs per SM
-// (40 registers, a few per-chunk values in local memory) keep more loads in
-// flight than the 64 registers the compiler picks unbounded (0.170 against
-// 0.200 ms per launch on 256 uneven problems; capping the registers with a
-// shallower unroll instead of spilling ran 0.32 ms).
+//
+// In 3D the loop streams the rows: registers are capped for 32 warps per SM
+// and eight loads deep (0.324 -> 0.277 ms per launch on a 64^3 porous level,
+// 1.29 GB, 8 lanes; 86 registers and 14 warps before).  A warp per patch takes
+// f_apply_stream_kernel.
+//
+// In 2D the patches of a chunk are split into those of the segment's two
+// class blocks and the others.  The class blocks are staged in shared memory
+// and each class patch is one thread's: rows by broadcast, residual loads by
+// consecutive lanes, no shuffles and no index arithmetic per slot; with 16
+// lanes per patch a warp took 306 instructions for two patches and the L1 was
+// 70 % busy (0.080 -> 0.035 to 0.044 ms on 48 problems of 64^2 to 111^2, 253
+// thousand patches).  Both ways add in the same order and round omega y
+// before the sum, so a patch's result does not depend on its way.  In 3D the
+// same split made the rows' stream thinner: a 96^3 solve took 90.7 ms with it
+// and 83.1 without.
 template <int DIM, int PT, int TPP>
-__global__ void __launch_bounds__(512, DIM == 2 ? 3 : 1)
+__global__ void __launch_bounds__(512, 2)
     f_apply_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
                    const int* __restrict__ state, int gate) {
   constexpr int ND = DIM + 1, NSLOT = DIM == 3 ? 402 : 59;
+  constexpr bool SPLIT = DIM == 2;
   using RL = RowLoad<PT, ND>;
   using T = typename RL::T;
   __shared__ int soff[NSLOT];
-  int cur_px = -1, cur_py = -1;
+  __shared__ float4 srow[SPLIT ? 2 * NSLOT : 1];
+  __shared__ unsigned short list[SPLIT ? kChunk : 1];  // class patches from the front, the others from the back
+  __shared__ int count[2];
+  int cur_seg = -1;
   const int lane = threadIdx.x % TPP, grp = threadIdx.x / TPP, ngrp = blockDim.x / TPP;
-  for (int c = blockIdx.x; c < nch; c += gridDim.x) {
-    const Chunk k = ch[c];
+  const int parts = apply_parts<DIM>(nch, ngrp), per = kChunk / parts;
+  for (int c = blockIdx.x; c < nch * parts; c += gridDim.x) {
+    Chunk k = ch[c / parts];
+    k.node0 += c % parts * per;
     const BSeg* S = segs + k.seg;
     if (state && state[S->prob] != gate) continue;  // uniform over the CTA
     const BGeom g = S->g;
-    const int px = g.nn[0] + 4, py = g.nn[1] + 4;
-    if (px != cur_px || py != cur_py) {
-      __syncthreads();
-      for (int j = threadIdx.x; j < NSLOT; j += blockDim.x) soff[j] = slot_offset<DIM>(j, px, py);
-      __syncthreads();
-      cur_px = px;
-      cur_py = py;
-    }
     const T* __restrict__ coef = static_cast<const T*>(S->coef);
     const int* __restrict__ prow = S->prow;
+    const int nq = (int)min((long long)per, g.nnodes - (long long)k.node0);
+    if (nq <= 0) continue;
+    int ncls = 0, noth = nq;
+    if (SPLIT || k.seg != cur_seg) {
+      __syncthreads();  // the chunk before is done with the tables
+      const int px = g.nn[0] + 4, py = g.nn[1] + 4, cls0 = S->cls[0], cls1 = S->cls[1];
+      if (k.seg != cur_seg) {
+        for (int j = threadIdx.x; j < NSLOT; j += blockDim.x) soff[j] = slot_offset<DIM>(j, px, py);
+        if constexpr (SPLIT)
+          for (int j = threadIdx.x; j < 2 * NSLOT; j += blockDim.x) {
+            const int blk = j < NSLOT ? cls0 : cls1, jj = j < NSLOT ? j : j - NSLOT;
+            float cv[ND] = {0.0f, 0.0f, 0.0f};
+            if (blk >= 0) RL::load(coef + ((size_t)blk * NSLOT + jj) * ND, true, cv);
+            srow[j] = make_float4(cv[0], cv[1], cv[2], __int_as_float(slot_offset<DIM>(jj, px, py)));
+          }
+        cur_seg = k.seg;
+      }
+      if constexpr (SPLIT) {
+        if (threadIdx.x < 2) count[threadIdx.x] = 0;
+        __syncthreads();
+        for (int q0 = 0; q0 < per; q0 += blockDim.x) {
+          const int q = q0 + threadIdx.x, wl = threadIdx.x & 31;
+          const int pr = q < nq && prow ? prow[k.node0 + q] : 0;
+          const bool of_class = pr < 0 && (-pr - 1 == cls0 || -pr - 1 == cls1);
+          const unsigned mc = __ballot_sync(0xffffffffu, of_class);
+          const unsigned mo = __ballot_sync(0xffffffffu, q < nq && !of_class);
+          int base = 0;
+          if (wl == 0 && mc) base = atomicAdd(&count[0], __popc(mc));
+          if (wl == 1 && mo) base = atomicAdd(&count[1], __popc(mo));
+          const int bc = __shfl_sync(0xffffffffu, base, 0), bo = __shfl_sync(0xffffffffu, base, 1);
+          const unsigned below = (1u << wl) - 1;
+          if (of_class)
+            list[bc + __popc(mc & below)] = (unsigned short)(-pr - 1 == cls0 ? q : q + kChunk);
+          else if (q < nq)
+            list[kChunk - 1 - bo - __popc(mo & below)] = (unsigned short)q;
+        }
+      }
+      __syncthreads();
+      if constexpr (SPLIT) {
+        ncls = count[0];
+        noth = count[1];
+      }
+    }
     const unsigned char* __restrict__ mask = S->mask;
     const float* __restrict__ rpad = S->rpadf;
     float* d = S->d32;
     const float omega = S->omega_f;
-    for (int q = grp; q < kChunk; q += ngrp) {
-      const long long node = (long long)k.node0 + q;
-      const bool valid = node < g.nnodes;
-      const unsigned i = (unsigned)(valid ? node : g.nnodes - 1);
+    for (int e0 = 0; e0 < noth; e0 += ngrp) {
+      const bool valid = e0 + grp < noth;
+      const int e = valid ? e0 + grp : noth - 1;
+      const unsigned i = (unsigned)k.node0 + (SPLIT ? list[kChunk - 1 - e] : e);
       int ia[3];
       decode(g, DIM, i, ia);
       const long long pb = padded(g, DIM, ia) * ND;
@@ -660,11 +761,11 @@ __global__ void __launch_bounds__(512, DIM == 2 ? 3 : 1)
       float y[ND];
 #pragma unroll
       for (int t = 0; t < ND; ++t) y[t] = 0.0f;
-#pragma unroll 4
+#pragma unroll 8
       for (int j = lane; j < NSLOT; j += TPP) {
         const float rv = rp[soff[j]];
         float cv[ND];
-        RL::load(cf + (size_t)j * ND, shared_rows, cv);
+        RL::load(cf + j * ND, SPLIT || shared_rows, cv);  // 2D: rows of 12 bytes share sectors, so cached
 #pragma unroll
         for (int t = 0; t < ND; ++t) y[t] = fmaf(cv[t], rv, y[t]);
       }
@@ -683,10 +784,156 @@ __global__ void __launch_bounds__(512, DIM == 2 ? 3 : 1)
           for (int u = 1; u < ND; ++u)
             if (t == u) yl = y[u];
           const bool fixed = t < DIM && ((mi >> t) & 1);
-          d[pb + t] += fixed ? rp[t] : omega * yl;
+          d[pb + t] = __fadd_rn(d[pb + t], fixed ? rp[t] : __fmul_rn(omega, yl));
         }
       }
     }
+    if constexpr (SPLIT)
+      for (int e = threadIdx.x; e < ncls; e += blockDim.x) {
+        const int le = list[e];
+        const unsigned i = (unsigned)k.node0 + (le & (kChunk - 1));
+        int ia[3];
+        decode(g, DIM, i, ia);
+        const long long pb = padded(g, DIM, ia) * ND;
+        const float* rp = rpad + pb;
+        float y[ND];
+        class_tree2<TPP, 1, 0>(srow + (le & kChunk ? NSLOT : 0), rp, y);
+        const unsigned char mi = mask[i];
+#pragma unroll
+        for (int t = 0; t < ND; ++t) {
+          const bool fixed = t < DIM && ((mi >> t) & 1);
+          d[pb + t] = __fadd_rn(d[pb + t], fixed ? rp[t] : __fmul_rn(omega, y[t]));
+        }
+      }
+  }
+}
+
+// The 3D apply with a warp per patch: the 402 rows of a patch with rows of its
+// own are copied to shared memory by cp.async while the patch before is
+// summed, so a warp always has 6.4 KB on the way; the plain loop left gaps
+// between patches.  0.259 -> 0.238 ms per launch on a 64^3 porous level
+// (1.29 GB: 5.4 TB/s, 79 % of the measured copy rate; the rest is the last
+// patches of uneven chunks) and 0.0145 -> 0.009 ms on its 17^3 level, where
+// the latency of one patch counts.  16 warps per SM at 128 registers: the 13
+// residual loads of a patch are all in flight while its rows arrive.  A lane
+// copies the rows that it will read itself, so its own wait is enough.  Class
+// rows are read through the caches.  Lanes, slots and order of sums as in
+// f_apply_kernel with 32 lanes.
+template <int RB>
+__device__ __forceinline__ void copy_row(void* dst, const void* src) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(dst);
+  if (RB == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(src) : "memory");
+}
+
+size_t stream_smem(fc_prec prec, int threads) {
+  return (size_t)(threads / 32) * 2 * 402 * (prec == FC_PREC_FP32 ? 16 : 8);
+}
+
+template <int PT>
+__global__ void __launch_bounds__(512, 1)
+    f_apply_stream_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
+                          const int* __restrict__ state, int gate) {
+  constexpr int ND = 4, NSLOT = 402, NI = (NSLOT + 31) / 32;
+  using RL = RowLoad<PT, ND>;
+  using T = typename RL::T;
+  constexpr int RB = ND * (int)sizeof(T);
+  extern __shared__ __align__(16) unsigned char stage_shm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  T* const buf = reinterpret_cast<T*>(stage_shm) + (size_t)warp * 2 * NSLOT * ND + lane * ND;
+  int cur_px = -1, cur_py = -1;
+  int off[NI];
+#pragma unroll
+  for (int u = 0; u < NI; ++u) off[u] = 0;
+  const int parts = apply_parts<3>(nch, nwarp), per = kChunk / parts;
+  for (int c = blockIdx.x; c < nch * parts; c += gridDim.x) {
+    Chunk k = ch[c / parts];
+    k.node0 += c % parts * per;
+    const BSeg* S = segs + k.seg;
+    if (state && state[S->prob] != gate) continue;
+    const BGeom g = S->g;
+    const int px = g.nn[0] + 4, py = g.nn[1] + 4;
+    if (px != cur_px || py != cur_py) {
+#pragma unroll
+      for (int u = 0; u < NI; ++u)
+        if (lane + 32 * u < NSLOT) off[u] = slot_offset<3>(lane + 32 * u, px, py);
+      cur_px = px;
+      cur_py = py;
+    }
+    const T* __restrict__ coef = static_cast<const T*>(S->coef) + lane * ND;
+    const unsigned char* __restrict__ mask = S->mask;
+    const float* __restrict__ rpad = S->rpadf;
+    float* d = S->d32;
+    const float omega = S->omega_f;
+    const int nq = (int)min((long long)per, g.nnodes - (long long)k.node0);
+    // this warp's patches: warp, warp + nwarp, ... (32 at most), lane e holds
+    // the row block of the e-th
+    const int mine = warp < nq ? (nq - warp + nwarp - 1) / nwarp : 0;
+    const int i0 = k.node0 + warp;
+    const int prl = lane < mine ? (S->prow ? S->prow[i0 + lane * nwarp] : i0 + lane * nwarp) : -1;
+    auto fetch = [&](int e) {
+      const int pr = __shfl_sync(0xffffffffu, prl, e);
+      if (e < mine && pr >= 0) {
+        const T* src = coef + (size_t)pr * NSLOT * ND;
+        T* dst = buf + (e & 1) * NSLOT * ND;
+#pragma unroll
+        for (int u = 0; u < NI; ++u)
+          if (u < NI - 1 || lane + 32 * u < NSLOT) copy_row<RB>(dst + 32 * u * ND, src + 32 * u * ND);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(0);
+    for (int e = 0; e < mine; ++e) {
+      fetch(e + 1);
+      const int i = i0 + e * nwarp;
+      int ia[3];
+      decode(g, 3, (unsigned)i, ia);
+      const long long pb = padded(g, 3, ia) * ND;
+      const float* rp = rpad + pb;
+      float rv[NI];
+#pragma unroll
+      for (int u = 0; u < NI; ++u) rv[u] = u < NI - 1 || lane + 32 * u < NSLOT ? rp[off[u]] : 0.0f;
+      const int t = lane >> 3;  // the component this lane's octet ends up with
+      const bool writer = (lane & 7) == 0;
+      const float dold = writer ? d[pb + t] : 0.0f, rself = writer ? rp[t] : 0.0f;
+      const unsigned char mi = mask[i];
+      const int pr = __shfl_sync(0xffffffffu, prl, e);
+      float y[ND] = {0.0f, 0.0f, 0.0f, 0.0f};
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      const T* rows = pr < 0 ? coef + (size_t)(-pr - 1) * NSLOT * ND : buf + (e & 1) * NSLOT * ND;
+      if (pr < 0) {
+#pragma unroll
+        for (int u = 0; u < NI; ++u)
+          if (u < NI - 1 || lane + 32 * u < NSLOT) {
+            float cv[ND];
+            RL::load(rows + 32 * u * ND, true, cv);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) y[q] = fmaf(cv[q], rv[u], y[q]);
+          }
+      } else {
+#pragma unroll
+        for (int u = 0; u < NI; ++u)
+          if (u < NI - 1 || lane + 32 * u < NSLOT) {
+            float cv[ND];
+            RL::load_shared(rows + 32 * u * ND, cv);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) y[q] = fmaf(cv[q], rv[u], y[q]);
+          }
+      }
+      const bool h1 = lane & 16, h2 = lane & 8;
+      float k0 = h1 ? y[2] : y[0], k1 = h1 ? y[3] : y[1];
+      k0 += __shfl_xor_sync(0xffffffffu, h1 ? y[0] : y[2], 16);
+      k1 += __shfl_xor_sync(0xffffffffu, h1 ? y[1] : y[3], 16);
+      float yl = h2 ? k1 : k0;
+      yl += __shfl_xor_sync(0xffffffffu, h2 ? k0 : k1, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) yl += __shfl_xor_sync(0xffffffffu, yl, o);
+      if (writer) {
+        const bool fixed = t < 3 && ((mi >> t) & 1);
+        d[pb + t] = __fadd_rn(dold, fixed ? rself : __fmul_rn(omega, yl));
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
 }
 
@@ -1314,8 +1561,10 @@ ApplyFn fapply_fn(int tpp) {
     case 4: return f_apply_kernel<DIM, PT, 4>;
     case 8: return f_apply_kernel<DIM, PT, 8>;
     case 16: return f_apply_kernel<DIM, PT, 16>;
-    default: return f_apply_kernel<DIM, PT, 32>;
+    default: break;
   }
+  if constexpr (DIM == 3) return f_apply_stream_kernel<PT>;
+  else return f_apply_kernel<DIM, PT, 32>;
 }
 
 template <int DIM, int PT>
@@ -1466,8 +1715,17 @@ fc_status apply(fc_batch B, const Plan& p, const Tile& t, const int* state, int 
     return FC_OK;
   }
   ApplyFn fn = pick_apply(B->dim, B->prec, t.tpp);
-  const unsigned grid = grid_of(B, p, t.ctas_per_sm);
-  fn<<<grid, t.threads, 0, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate);
+  Plan items = p;
+  if (B->f32) items.count *= B->dim == 3 ? apply_parts<3>(p.count, t.threads / t.tpp) : apply_parts<2>(p.count, t.threads / t.tpp);
+  size_t smem = 0;
+  int per_sm = t.ctas_per_sm, nsm = 0;
+  if (B->f32 && B->dim == 3 && t.tpp == 32) {
+    smem = stream_smem(B->prec, t.threads);
+    BK(persistent_ctas((const void*)fn, t.threads, smem, &per_sm, &nsm));
+    per_sm = std::min(per_sm, t.ctas_per_sm);
+  }
+  const unsigned grid = grid_of(B, items, per_sm);
+  fn<<<grid, t.threads, smem, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate);
   note_launches(1);
   BK(cudaGetLastError());
   return FC_OK;
