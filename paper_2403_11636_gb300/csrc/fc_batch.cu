@@ -270,7 +270,7 @@ __device__ __forceinline__ int slot_offset(int j, int px, int py) {
 template <int DIM, int PT, int TPP>
 __global__ void __launch_bounds__(512)
     b_apply_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
-                   const int* __restrict__ state, int gate) {
+                   const int* __restrict__ state, int gate, int /*split*/) {
   constexpr int ND = DIM + 1, NSLOT = DIM == 3 ? 402 : 59;
   using RL = RowLoad<PT, ND>;
   using T = typename RL::T;
@@ -555,13 +555,14 @@ __device__ __forceinline__ void load_node(const float* p, float* v) {
 }
 
 // r = b32 - L32 d into the padded float32 residual.  Bound by the latency of
-// its loads: half a chunk per CTA and registers for 32 warps per SM, so that
-// coarse levels and the last CTAs of a fine one spread over more SMs.  64^3
-// level 0.053 -> 0.042 ms (123 MB of stencil, 0.018 ms at the copy rate), 48 2D
-// problems 0.421 -> 0.338 ms per two V-cycles.
+// its loads: half a chunk per CTA and registers for 28 (3D) or 32 warps per SM, so
+// that coarse levels and the last CTAs of a fine one spread over more SMs.  64^3
+// level 0.053 -> 0.051 ms (123 MB of stencil, 0.018 ms at the copy rate; 0.042
+// with 64 registers, but then it spills), 48 2D problems 0.421 -> 0.338 ms per
+// two V-cycles.
 constexpr int kHalf = kChunk / 2;
 template <int DIM>
-__global__ void __launch_bounds__(kHalf, 8)
+__global__ void __launch_bounds__(kHalf, DIM == 3 ? 7 : 8)
     f_residual_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
                       const int* __restrict__ state, int gate) {
   // half stencil: the zero offset and the offsets after it are the node's
@@ -636,137 +637,55 @@ __global__ void __launch_bounds__(kHalf, 8)
   }
 }
 
-// One 2D patch's product by one thread, in the order of the TPP-lane sum: a
-// leaf (S == TPP) is lane LANE's, the slots LANE, LANE + TPP, ..., then the
-// lanes are added pairwise (l with l + TPP/2 first).  Depth first, so no more
-// than log2(TPP) + 1 partial rows are live.  A row's fourth float is the bits
-// of its slot's offset.
-template <int TPP, int S, int LANE>
-__device__ __forceinline__ void class_tree2(const float4* rows, const float* rp, float* y) {
-  constexpr int NSLOT = 59;
-  if constexpr (S == TPP) {
-    y[0] = y[1] = y[2] = 0.0f;
-#pragma unroll
-    for (int j = LANE; j < NSLOT; j += TPP) {
-      const float4 cv = rows[j];
-      const float rv = rp[__float_as_int(cv.w)];
-      y[0] = fmaf(cv.x, rv, y[0]);
-      y[1] = fmaf(cv.y, rv, y[1]);
-      y[2] = fmaf(cv.z, rv, y[2]);
-    }
-  } else {
-    float b[3];
-    class_tree2<TPP, 2 * S, LANE>(rows, rp, y);
-    class_tree2<TPP, 2 * S, LANE + S>(rows, rp, b);
-#pragma unroll
-    for (int t = 0; t < 3; ++t) y[t] += b[t];
-  }
-}
-
-// Parts of a chunk in the float32 applies, for levels with too few chunks to
-// fill the SMs evenly: with whole chunks a 33^3 level ran 0.127 ms and a 17^3
-// level as long (every group had the same 8 patches in sequence), with parts
-// 0.047 and 0.009 ms (3D, float32 rows).  In 2D a part costs its own split
-// into class and other patches: 1216 and more items were slower on 48
-// problems of 64^2 to 111^2 (0.031 against 0.028 ms on their second level).
-template <int DIM>
-__host__ __device__ constexpr int apply_parts(int nch, int ngrp) {
-  int parts = kChunk > 32 * ngrp ? kChunk / (32 * ngrp) : 1;  // 32 patches a group at most
-  while (2 * parts * ngrp <= kChunk && (long long)nch * parts < (DIM == 3 ? 2432 : 608)) parts *= 2;
-  return parts;
-}
-
 // d += omega L_i^{-1} r on the owned DoFs (PT 1: float32 rows, 2: bfloat16).
+//
+// The 2D loop is bound by the latency of its loads (rows from the cache for
+// the shared class blocks, residual gathers): three 512-thread CTAs per SM
+// (40 registers, a few per-chunk values in local memory) keep more loads in
+// flight than the 64 registers the compiler picks unbounded (0.170 against
+// 0.200 ms per launch on 256 uneven problems; capping the registers with a
+// shallower unroll instead of spilling ran 0.32 ms; 0.156 with every row load
+// cached, for the flag made two loads of each).  Class patches apart, a
+// thread each with the class rows in shared memory, ran 0.181 to 0.188 ms.
 //
 // In 3D the loop streams the rows: registers are capped for 32 warps per SM
 // and eight loads deep (0.324 -> 0.277 ms per launch on a 64^3 porous level,
 // 1.29 GB, 8 lanes; 86 registers and 14 warps before).  A warp per patch takes
 // f_apply_stream_kernel.
-//
-// In 2D the patches of a chunk are split into those of the segment's two
-// class blocks and the others.  The class blocks are staged in shared memory
-// and each class patch is one thread's: rows by broadcast, residual loads by
-// consecutive lanes, no shuffles and no index arithmetic per slot; with 16
-// lanes per patch a warp took 306 instructions for two patches and the L1 was
-// 70 % busy (0.080 -> 0.035 to 0.044 ms on 48 problems of 64^2 to 111^2, 253
-// thousand patches).  Both ways add in the same order and round omega y
-// before the sum, so a patch's result does not depend on its way.  In 3D the
-// same split made the rows' stream thinner: a 96^3 solve took 90.7 ms with it
-// and 83.1 without.
 template <int DIM, int PT, int TPP>
-__global__ void __launch_bounds__(512, 2)
+__global__ void __launch_bounds__(512, DIM == 2 ? 3 : 2)
     f_apply_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
-                   const int* __restrict__ state, int gate) {
+                   const int* __restrict__ state, int gate, int split) {
   constexpr int ND = DIM + 1, NSLOT = DIM == 3 ? 402 : 59;
-  constexpr bool SPLIT = DIM == 2;
   using RL = RowLoad<PT, ND>;
   using T = typename RL::T;
   __shared__ int soff[NSLOT];
-  __shared__ float4 srow[SPLIT ? 2 * NSLOT : 1];
-  __shared__ unsigned short list[SPLIT ? kChunk : 1];  // class patches from the front, the others from the back
-  __shared__ int count[2];
-  int cur_seg = -1;
+  int cur_px = -1, cur_py = -1;
   const int lane = threadIdx.x % TPP, grp = threadIdx.x / TPP, ngrp = blockDim.x / TPP;
-  const int parts = apply_parts<DIM>(nch, ngrp), per = kChunk / parts;
-  for (int c = blockIdx.x; c < nch * parts; c += gridDim.x) {
-    Chunk k = ch[c / parts];
-    k.node0 += c % parts * per;
+  for (int c = blockIdx.x; c < nch << split; c += gridDim.x) {
+    Chunk k = ch[c >> split];
+    k.node0 += (c & ((1 << split) - 1)) * (kChunk >> split);
     const BSeg* S = segs + k.seg;
     if (state && state[S->prob] != gate) continue;  // uniform over the CTA
     const BGeom g = S->g;
+    const int px = g.nn[0] + 4, py = g.nn[1] + 4;
+    if (px != cur_px || py != cur_py) {
+      __syncthreads();
+      for (int j = threadIdx.x; j < NSLOT; j += blockDim.x) soff[j] = slot_offset<DIM>(j, px, py);
+      __syncthreads();
+      cur_px = px;
+      cur_py = py;
+    }
     const T* __restrict__ coef = static_cast<const T*>(S->coef);
     const int* __restrict__ prow = S->prow;
-    const int nq = (int)min((long long)per, g.nnodes - (long long)k.node0);
-    if (nq <= 0) continue;
-    int ncls = 0, noth = nq;
-    if (SPLIT || k.seg != cur_seg) {
-      __syncthreads();  // the chunk before is done with the tables
-      const int px = g.nn[0] + 4, py = g.nn[1] + 4, cls0 = S->cls[0], cls1 = S->cls[1];
-      if (k.seg != cur_seg) {
-        for (int j = threadIdx.x; j < NSLOT; j += blockDim.x) soff[j] = slot_offset<DIM>(j, px, py);
-        if constexpr (SPLIT)
-          for (int j = threadIdx.x; j < 2 * NSLOT; j += blockDim.x) {
-            const int blk = j < NSLOT ? cls0 : cls1, jj = j < NSLOT ? j : j - NSLOT;
-            float cv[ND] = {0.0f, 0.0f, 0.0f};
-            if (blk >= 0) RL::load(coef + ((size_t)blk * NSLOT + jj) * ND, true, cv);
-            srow[j] = make_float4(cv[0], cv[1], cv[2], __int_as_float(slot_offset<DIM>(jj, px, py)));
-          }
-        cur_seg = k.seg;
-      }
-      if constexpr (SPLIT) {
-        if (threadIdx.x < 2) count[threadIdx.x] = 0;
-        __syncthreads();
-        for (int q0 = 0; q0 < per; q0 += blockDim.x) {
-          const int q = q0 + threadIdx.x, wl = threadIdx.x & 31;
-          const int pr = q < nq && prow ? prow[k.node0 + q] : 0;
-          const bool of_class = pr < 0 && (-pr - 1 == cls0 || -pr - 1 == cls1);
-          const unsigned mc = __ballot_sync(0xffffffffu, of_class);
-          const unsigned mo = __ballot_sync(0xffffffffu, q < nq && !of_class);
-          int base = 0;
-          if (wl == 0 && mc) base = atomicAdd(&count[0], __popc(mc));
-          if (wl == 1 && mo) base = atomicAdd(&count[1], __popc(mo));
-          const int bc = __shfl_sync(0xffffffffu, base, 0), bo = __shfl_sync(0xffffffffu, base, 1);
-          const unsigned below = (1u << wl) - 1;
-          if (of_class)
-            list[bc + __popc(mc & below)] = (unsigned short)(-pr - 1 == cls0 ? q : q + kChunk);
-          else if (q < nq)
-            list[kChunk - 1 - bo - __popc(mo & below)] = (unsigned short)q;
-        }
-      }
-      __syncthreads();
-      if constexpr (SPLIT) {
-        ncls = count[0];
-        noth = count[1];
-      }
-    }
     const unsigned char* __restrict__ mask = S->mask;
     const float* __restrict__ rpad = S->rpadf;
     float* d = S->d32;
     const float omega = S->omega_f;
-    for (int e0 = 0; e0 < noth; e0 += ngrp) {
-      const bool valid = e0 + grp < noth;
-      const int e = valid ? e0 + grp : noth - 1;
-      const unsigned i = (unsigned)k.node0 + (SPLIT ? list[kChunk - 1 - e] : e);
+    for (int q = grp; q < kChunk >> split; q += ngrp) {
+      const long long node = (long long)k.node0 + q;
+      const bool valid = node < g.nnodes;
+      const unsigned i = (unsigned)(valid ? node : g.nnodes - 1);
       int ia[3];
       decode(g, DIM, i, ia);
       const long long pb = padded(g, DIM, ia) * ND;
@@ -777,11 +696,12 @@ __global__ void __launch_bounds__(512, 2)
       float y[ND];
 #pragma unroll
       for (int t = 0; t < ND; ++t) y[t] = 0.0f;
-#pragma unroll 8
+#pragma unroll(DIM == 3 ? 8 : 4)
       for (int j = lane; j < NSLOT; j += TPP) {
         const float rv = rp[soff[j]];
         float cv[ND];
-        RL::load(cf + j * ND, SPLIT || shared_rows, cv);  // 2D: rows of 12 bytes share sectors, so cached
+        // 2D: rows of 12 bytes share sectors, so they are cached in any case
+        RL::load(cf + (size_t)j * ND, DIM == 2 || shared_rows, cv);
 #pragma unroll
         for (int t = 0; t < ND; ++t) y[t] = fmaf(cv[t], rv, y[t]);
       }
@@ -804,23 +724,6 @@ __global__ void __launch_bounds__(512, 2)
         }
       }
     }
-    if constexpr (SPLIT)
-      for (int e = threadIdx.x; e < ncls; e += blockDim.x) {
-        const int le = list[e];
-        const unsigned i = (unsigned)k.node0 + (le & (kChunk - 1));
-        int ia[3];
-        decode(g, DIM, i, ia);
-        const long long pb = padded(g, DIM, ia) * ND;
-        const float* rp = rpad + pb;
-        float y[ND];
-        class_tree2<TPP, 1, 0>(srow + (le & kChunk ? NSLOT : 0), rp, y);
-        const unsigned char mi = mask[i];
-#pragma unroll
-        for (int t = 0; t < ND; ++t) {
-          const bool fixed = t < DIM && ((mi >> t) & 1);
-          d[pb + t] = __fadd_rn(d[pb + t], fixed ? rp[t] : __fmul_rn(omega, y[t]));
-        }
-      }
   }
 }
 
@@ -849,7 +752,7 @@ size_t stream_smem(fc_prec prec, int threads) {
 template <int PT>
 __global__ void __launch_bounds__(512, 1)
     f_apply_stream_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
-                          const int* __restrict__ state, int gate) {
+                          const int* __restrict__ state, int gate, int split) {
   constexpr int ND = 4, NSLOT = 402, NI = (NSLOT + 31) / 32;
   using RL = RowLoad<PT, ND>;
   using T = typename RL::T;
@@ -861,10 +764,9 @@ __global__ void __launch_bounds__(512, 1)
   int off[NI];
 #pragma unroll
   for (int u = 0; u < NI; ++u) off[u] = 0;
-  const int parts = apply_parts<3>(nch, nwarp), per = kChunk / parts;
-  for (int c = blockIdx.x; c < nch * parts; c += gridDim.x) {
-    Chunk k = ch[c / parts];
-    k.node0 += c % parts * per;
+  for (int c = blockIdx.x; c < nch << split; c += gridDim.x) {
+    Chunk k = ch[c >> split];
+    k.node0 += (c & ((1 << split) - 1)) * (kChunk >> split);
     const BSeg* S = segs + k.seg;
     if (state && state[S->prob] != gate) continue;
     const BGeom g = S->g;
@@ -881,7 +783,7 @@ __global__ void __launch_bounds__(512, 1)
     const float* __restrict__ rpad = S->rpadf;
     float* d = S->d32;
     const float omega = S->omega_f;
-    const int nq = (int)min((long long)per, g.nnodes - (long long)k.node0);
+    const int nq = (int)min((long long)(kChunk >> split), g.nnodes - (long long)k.node0);
     // this warp's patches: warp, warp + nwarp, ... (32 at most), lane e holds
     // the row block of the e-th
     const int mine = warp < nq ? (nq - warp + nwarp - 1) / nwarp : 0;
@@ -1037,7 +939,7 @@ __global__ void tc_prepare_kernel(const T* __restrict__ coef, int cls0, int cls1
 template <int DIM, int PT, int MODE>
 __global__ void __launch_bounds__(256)
     f_apply_tc_kernel(const BSeg* __restrict__ segs, const Chunk* __restrict__ ch, int nch,
-                      const int* __restrict__ state, int gate) {
+                      const int* __restrict__ state, int gate, int /*split*/) {
   using D = TcDims<DIM>;
   constexpr int ND = DIM + 1, NSLOT = D::NSLOT, KP = D::KP;
   using RL = RowLoad<PT, ND>;
@@ -1583,7 +1485,7 @@ struct Tile {
   int tpp = 16, threads = 256, ctas_per_sm = 8;
 };
 
-typedef void (*ApplyFn)(const BSeg*, const Chunk*, int, const int*, int);
+typedef void (*ApplyFn)(const BSeg*, const Chunk*, int, const int*, int, int);
 
 template <int DIM, int PT>
 ApplyFn apply_fn(int tpp) {
@@ -1609,6 +1511,20 @@ ApplyFn fapply_fn(int tpp) {
   }
   if constexpr (DIM == 3) return f_apply_stream_kernel<PT>;
   else return f_apply_kernel<DIM, PT, 32>;
+}
+
+// The float32 applies split every chunk into 2^this parts, for levels with too
+// few chunks to fill the SMs evenly: with whole chunks a 33^3 level ran 0.127
+// ms and a 17^3 level as long (every group had the same 8 patches one after
+// the other), with parts 0.047 and 0.009 ms (3D, float32 rows); the second and
+// third levels of 48 2D problems 0.027 -> 0.017 and 0.009 ms.  2,432 items are
+// two waves of eight CTAs per SM.  A part is a kernel argument, so that it
+// costs the kernels no register.
+int apply_split(int nch, int ngrp) {
+  int s = 0;
+  while (kChunk >> s > 32 * ngrp) ++s;  // 32 patches a group at most
+  while (kChunk >> (s + 1) >= ngrp && ((long long)nch << s) < 2432) ++s;
+  return s;
 }
 
 template <int DIM, int PT>
@@ -1753,14 +1669,15 @@ fc_status apply(fc_batch B, const Plan& p, const Tile& t, const int* state, int 
     const size_t smem = tc_smem(B->dim, B->tc);
     int per_sm = 0, nsm = 0;
     BK(persistent_ctas((const void*)fn, 256, smem, &per_sm, &nsm));
-    fn<<<grid_of(B, p, per_sm), 256, smem, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate);
+    fn<<<grid_of(B, p, per_sm), 256, smem, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate, 0);
     note_launches(1);
     BK(cudaGetLastError());
     return FC_OK;
   }
   ApplyFn fn = pick_apply(B->dim, B->prec, t.tpp);
   Plan items = p;
-  if (B->f32) items.count *= B->dim == 3 ? apply_parts<3>(p.count, t.threads / t.tpp) : apply_parts<2>(p.count, t.threads / t.tpp);
+  const int split = B->f32 ? apply_split(p.count, t.threads / t.tpp) : 0;
+  items.count <<= split;
   size_t smem = 0;
   int per_sm = t.ctas_per_sm, nsm = 0;
   if (B->f32 && B->dim == 3 && t.tpp == 32) {
@@ -1769,7 +1686,7 @@ fc_status apply(fc_batch B, const Plan& p, const Tile& t, const int* state, int 
     per_sm = std::min(per_sm, t.ctas_per_sm);
   }
   const unsigned grid = grid_of(B, items, per_sm);
-  fn<<<grid, t.threads, smem, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate);
+  fn<<<grid, t.threads, smem, B->s>>>(B->segs, B->chunks + p.first, p.count, state, gate, split);
   note_launches(1);
   BK(cudaGetLastError());
   return FC_OK;
