@@ -16,7 +16,8 @@ instrumented).  Per-kernel times for the roofline come from a separate pass
 of profiled solves after the timed ones.  With FP64 rows the patch apply is
 bound by the FP64 pipe (GB300 runs FP64 at 1/64 of the FP32 rate), so its
 roofline is FP64 FLOP/s against the nominal pipe peak, with the live FMA
-probe and the HBM fraction beside it.
+probe and the HBM fraction beside it.  The operations counted are those of
+the FP64 pipe; uncut patches take the tensor cores (fc_digits.cu).
 
 --impl reference times the FP64 CPU oracle (the plain implementation the
 tests compare against) on the host cores, on a bounded sample of the same
@@ -288,8 +289,9 @@ def run_ours(args, rank, world, local_rank):
         n_fine, ms_fine, bytes_fine = s.profile_read(4)
         n_res, ms_res, _ = s.profile_read(1)
         n_vc, ms_vc, _ = s.profile_read(2)
-        s.profile(False)
         flops_fine = s.info()["bytes"][6]
+        _, _, flops_pipe = s.profile_read(5)
+        s.profile(False)
         # ---- end to end through the public API with host buffers
         n = s.ndof()
         bh = torch.empty(n, dtype=torch.float64, pin_memory=True)
@@ -322,7 +324,9 @@ def run_ours(args, rank, world, local_rank):
     hbm, peak_kind = peaks()
     avg_fine_ms = ms_fine / max(n_fine, 1)
     gbs = bytes_fine / (avg_fine_ms * 1e-3) / 1e9 if ms_fine > 0 else 0.0
-    tflops = flops_fine / (avg_fine_ms * 1e-3) / 1e12 if ms_fine > 0 else 0.0
+    # the FP64 pipe's share: uncut patches of large levels are multiplied on
+    # the tensor cores (exact digit products) in the same launches
+    tflops = flops_pipe / (avg_fine_ms * 1e-3) / 1e12 if ms_fine > 0 else 0.0
     traffic = load_traffic(args.prec) if not args.dedup else None
     if args.prec == "fp64":
         peak_tf, peak_note = fp64_peak(torch)
@@ -336,7 +340,7 @@ def run_ours(args, rank, world, local_rank):
                 "peak_source": peak_kind}
     roof.update({"kernel": "patch apply (cache_inverse) on the finest level", "launches": n_fine,
                  "avg_launch_ms": avg_fine_ms, "algorithmic_bytes_per_launch": bytes_fine,
-                 "algorithmic_flop_per_launch": flops_fine,
+                 "algorithmic_flop_per_launch": flops_fine, "fp64_pipe_flop_per_launch": flops_pipe,
                  "timing": f"CUDA events on the solver stream around every finest-level apply of "
                            f"{max(1, min(args.steps, args.profile_steps))} profiled solves after the timed ones"})
     out = {
@@ -751,10 +755,11 @@ def run_replay(args):
                 s.profile(True)
                 s.smooth_(X, b, nsweeps=10)
                 na, ma, ba = s.profile_read(4)
+                nf, _, flop = s.profile_read(5)  # the FP64 pipe's share
                 s.profile(False)
                 torch.cuda.synchronize()
                 avg = ma / max(na, 1)
-                flop = float(s.info()["bytes"][6])
+                flop = flop if nf else float(s.info()["bytes"][6])
                 tf, _ = fp64_peak(torch)
                 hbm, _ = peaks()
                 apply = {"ms": avg, "flop_per_launch": flop, "bytes_per_launch": ba,

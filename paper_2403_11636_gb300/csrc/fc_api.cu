@@ -278,12 +278,23 @@ LevelGeom make_geom(const fc_grid* g, int nshape, const Shape* d_shapes, double 
 
 namespace {
 
+double class_patches(const Level& L) { return (double)(L.g.nnodes - L.dig[0].nlist); }
+
 double level_apply_bytes(fc_handle h, int li) {
   const Level& L = h->lev[li];
   double cb = (double)coef_elem_bytes(h->opt.prec);
   double rb = (h->opt.prec == FC_PREC_FP32 || h->opt.prec == FC_PREC_BF16) ? 4.0 : 8.0;
   double act = (double)L.active_work;  // rows streamed: stored blocks, each once
+  // class patches on the tensor cores stream no rows of their own
+  if (L.dig[0].on && !h->opt.dedup) act -= class_patches(L) * nslot(L.g.dim);
   return act * L.g.nd * cb + (double)L.g.nnodes * L.g.nd * (rb + 16.0);
+}
+
+// floating-point operations of a patch apply on the FP64 pipe: all but the
+// class patches of fc_digits.cu (uncut and free: every slot and row active)
+double level_fp64_flop(const Level& L) {
+  const double all = 2.0 * (double)L.active_rows;
+  return L.dig[0].on ? all - 2.0 * class_patches(L) * nslot(L.g.dim) * L.g.nd : all;
 }
 
 // residual into the smoother's input buffer (format per precision)
@@ -380,6 +391,7 @@ fc_status smooth_level(fc_handle h, int li, double* x, const double* b, int nswe
     if (h->opt.cache == FC_CACHE_INVERSE) {
       ProfScope ps(h, 0, level_apply_bytes(h, li));
       ProfScope pf(h, li == h->nlev - 1 ? 4 : -1, level_apply_bytes(h, li));
+      ProfScope pw(h, li == h->nlev - 1 && h->opt.prec == FC_PREC_FP64 ? 5 : -1, level_fp64_flop(L));
       CK(apply_rows(L, h->opt.prec, L.rpad, L.rpad32, h->opt.omega, x, h->stream));
     } else if (h->opt.cache == FC_CACHE_MATRIX) {
       ProfScope ps(h, 0, (double)L.fac_bytes);
