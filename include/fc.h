@@ -46,6 +46,8 @@
  *    banded LDL^T of a 3D patch's velocity block accepts before the patch
  *    goes to the pivoted dense LU; a value above 1 sends every patch there
  *    (the two paths give the same rows up to rounding, which tests use).
+ *    FC_DIGIT_WAIT_NS (default 1e9) bounds the wait for the tensor-core
+ *    products of uncut nodes; past it a tile forms them in FP64 (0: at once).
  */
 #ifndef FC_H
 #define FC_H

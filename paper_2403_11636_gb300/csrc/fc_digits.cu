@@ -43,6 +43,7 @@
 // nodes, to the FP64 kernels (plan list).
 #include <cuda_fp16.h>
 #include <math.h>
+#include <stdlib.h>
 
 #include <algorithm>
 
@@ -139,12 +140,14 @@ __device__ __forceinline__ long long fixed_point(double v, int emax, int shift) 
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 // ---- tcgen05, mbarrier and bulk copies
-constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait that takes a second gives up
+// A wait gives up after a second (the wait for products after the plan's wait_ns)
+constexpr unsigned long long kWaitNs = 1000000000ull;
 
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, unsigned long long limit = kWaitNs) {
+  if (limit == 0ull) return false;
   unsigned long long start = 0ull;
   for (;;) {
     unsigned done;
@@ -157,7 +160,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
     if (start == 0ull) start = now;
-    else if (now - start > kWaitNs) return false;
+    else if (now - start > limit) return false;
   }
 }
 // global -> shared copy of `bytes` (a multiple of 16) that completes on bar
@@ -206,6 +209,7 @@ struct DigArgs {
   const double* w;
   const DigitScale* sc;
   unsigned* err;
+  unsigned long long wait_ns;
   const int* list;
   int nlist, list_blocks;
   // KIND 0: v = padded residual, x updated.  KIND 1: v = x, r and rpad
@@ -299,15 +303,18 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
   unsigned* soffs = reinterpret_cast<unsigned*>(smem + D::O_OFFS);
   unsigned char* scls = reinterpret_cast<unsigned char*>(smem + D::O_CLS);
   constexpr int NH = (D::NHALO + D::THREADS - 1) / D::THREADS;
-  // W arrived [NST], W used [NST], products done [per block where W is one piece]
+  // W arrived [NST], W used [NST], products done [per block where W is one
+  // piece], drained.  Every arrival is waited for before the CTA ends: a block
+  // without nodes of the class and a place that takes no further piece of W are
+  // not committed.
   constexpr int NDONE = D::NCH == 1 ? D::NBLK : 1;
-  __shared__ __align__(8) unsigned long long sbar[2 * D::NST + NDONE];
+  __shared__ __align__(8) unsigned long long sbar[2 * D::NST + NDONE + 1];
   __shared__ int semax[2], sbad, sfail;
   __shared__ unsigned sblk[2], stmem;
   const int tid = threadIdx.x, lane = tid & 31, wib = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const unsigned sbase = (unsigned)__cvta_generic_to_shared(smem);
   const unsigned bar0 = (unsigned)__cvta_generic_to_shared(sbar);
-  const unsigned bar_done = bar0 + 8 * 2 * D::NST;
+  const unsigned bar_done = bar0 + 8 * 2 * D::NST, bar_drain = bar_done + 8 * NDONE;
   const unsigned tile = blockIdx.x - (unsigned)a.list_blocks, tq = tile / (unsigned)tiles_x;
   // the first R layers of a grid hold no class node (their boxes leave it): of
   // 2^k + 1 nodes, a multiple of the tile and a remainder are left
@@ -339,7 +346,7 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
   const int delta[2] = {a.sc[0].delta, a.sc[1].delta};
   const bool sc_ok[2] = {a.sc[0].ok != 0, a.sc[1].ok != 0};
   if (tid == 0) {
-    for (int k = 0; k < 2 * D::NST + NDONE; ++k) mbar_init(bar0 + 8 * k, 1);
+    for (int k = 0; k < 2 * D::NST + NDONE + 1; ++k) mbar_init(bar0 + 8 * k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     semax[0] = semax[1] = -100000;
     sblk[0] = sblk[1] = 0u;
@@ -449,7 +456,13 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
   tc_fence_after();
   const unsigned tmem = stmem;
   int piece = 0;  // pieces of W so far: parities of their barriers
-  unsigned done = 0;
+  unsigned done = 0;  // parities of the barriers of products done, a bit each
+  unsigned owed = 0, owed_parity = 0;  // the issuing thread: barriers with a commit, a bit each
+  auto commit = [&](int b, unsigned parity) {
+    tc_commit(bar0 + 8 * b);
+    owed |= 1u << b;
+    owed_parity = (owed_parity & ~(1u << b)) | (parity << b);
+  };
   for (int cls = 1; cls <= 2; ++cls) {
     const unsigned blocks = sblk[cls - 1];
     if (blocks == 0u) continue;
@@ -467,7 +480,8 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
           const unsigned idesc = (1u << 4) | ((unsigned)(D::N >> 3) << 17) | ((128u >> 4) << 24);
           const unsigned a0 = sbase >> 4;
           bool ok = true;
-          int loaded = cls == first ? (D::NST < D::NCH ? D::NST : D::NCH) : 0;
+          const bool more = cls == 1 && sblk[1] != 0u && usable(2);  // class 2 takes the places next
+          int loaded = cls == first ? (D::NST < D::NCH ? D::NST : D::NCH) : 0, waited = 0;
           for (; loaded < D::NST && loaded < D::NCH; ++loaded) {
             const int p = piece + loaded;
             if (p >= D::NST)
@@ -488,6 +502,7 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
             }
             ok = ok && mbar_wait(bar0 + 8 * st, (unsigned)((p / D::NST) & 1));
             if (!ok) break;
+            ++waited;
             tc_fence_after();
             const unsigned b0 =
                 ((sbase + (unsigned)D::O_ROWS + st * D::CS * 1024) >> 4) | ((512u >> 4) << 16);
@@ -503,10 +518,9 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
                   for (int t = 0; t < D::STEPS; ++t)
                     tc_mma(tmem + blk * D::N, hi | (unsigned long long)(soffs[t] + (a0 + blk * 128)),
                            hi | (unsigned long long)(b0 + (unsigned)t * 64), idesc, t > 0);
+                  commit(2 * D::NST + blk, (done >> blk) & 1u);
                 }
-                tc_commit(bar_done + 8 * blk);
               }
-              tc_commit(bar0 + 8 * (D::NST + st));
             } else {
               unsigned so = soffs[t0] + a0;
 #pragma unroll 2
@@ -519,15 +533,16 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
                     tc_mma(tmem + blk * D::N, hi | (unsigned long long)(so + blk * 128), db, idesc, t > 0);
                 so = next;
               }
-              tc_commit(bar0 + 8 * (D::NST + st));
             }
+            if (more || k + D::NST < D::NCH) commit(D::NST + st, (p / D::NST) & 1);
           }
-          if (D::NCH > 1) tc_commit(bar_done);
+          if (D::NCH > 1 && ok) commit(2 * D::NST, done & 1u);
           if (!ok) {
             // give up: once more for the copies on their way; what waits for
-            // the products waits no longer than its own limit
+            // the products gives up at its own limit, the products on their way
+            // are waited for at the end
             sfail = 1;
-            for (int k = loaded > D::NST ? loaded - D::NST : 0; k < loaded; ++k)
+            for (int k = waited; k < loaded; ++k)
               mbar_wait(bar0 + 8 * ((piece + k) % D::NST), (unsigned)(((piece + k) / D::NST) & 1));
           }
         }
@@ -548,6 +563,7 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
 #pragma unroll
       for (int c = 0; c < ND; ++c) own[q][c] = from ? from[n * ND + c] : 0.0;
     }
+    bool gave_up = false;
     double scale[ND];
 #pragma unroll
     for (int n = 0; n < ND; ++n) {
@@ -561,18 +577,24 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
       const int m = blk * 128 + (wib & 3) * 32 + lane;
       const int ia[3] = {bx + m % D::HX, by + (DIM == 3 ? (m / D::HX) % D::HY : m / D::HX),
                          DIM == 3 ? bz + m / (D::HX * D::HY) : 0};
-      double y[ND];
-      bool fp64 = plain;
-      if (!fp64 && !mbar_wait(bar_done + 8 * (NDONE > 1 ? blk : 0), done & 1)) {
-        fp64 = true;  // no products: say so and form them in FP64
-        if (lane == 0) {
-          atomicOr(a.err, kErrTimeout);
-          sfail = 1;
-        }
+      double y[ND], sc[ND];
 #pragma unroll
-        for (int n = 0; n < ND; ++n) scale[n] = KIND == 0 ? a.omega : 1.0;
+      for (int n = 0; n < ND; ++n) sc[n] = scale[n];
+      bool fp64 = plain || gave_up;
+      if (!fp64) {
+        // (the warp agrees: tcgen05.ld needs all of it)
+        const int at = NDONE > 1 ? blk : 0;
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_done + 8 * at, (done >> at) & 1u, a.wait_ns))) {
+          fp64 = gave_up = true;  // no products: say so and form them in FP64, these and the warp's others
+          if (lane == 0) {
+            atomicOr(a.err, kErrTimeout);
+            sfail = 1;
+          }
+        }
       }
       if (fp64) {
+#pragma unroll
+        for (int n = 0; n < ND; ++n) sc[n] = KIND == 0 ? a.omega : 1.0;
         if (rc[q] == cls) fp64_product<DIM, KIND>(g, a.w + (size_t)(cls - 1) * D::NSLOT * ND, a.v, ia, y);
       } else {
         tc_fence_after();
@@ -594,9 +616,9 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
                  __longlong_as_double(0x4138000000000000ll + h[1]);
         }
       }
-      if (rc[q] == cls) store_product<DIM, KIND>(g, a, ia, own[q], y, scale);
+      if (rc[q] == cls) store_product<DIM, KIND>(g, a, ia, own[q], y, sc);
     }
-    if (!plain) done ^= 1;
+    if (!plain) done ^= NDONE > 1 ? blocks : 1u;
     if (cls == 1 && sblk[1] != 0u) {  // the accumulators are read before the other class's products
       tc_fence_before();
       __syncthreads();
@@ -605,6 +627,18 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 2 : 3)
   }
   tc_fence_before();
   __syncthreads();
+  if (sfail) {
+    // products may be on their way: the thread that issued them waits for them
+    // and for what its commits have not signalled yet, before tensor and shared
+    // memory are given back
+    if (wib == 0 && elect_one()) {
+      tc_commit(bar_drain);
+      mbar_wait(bar_drain, 0u);
+      for (int b = 0; b < 2 * D::NST + NDONE; ++b)
+        if ((owed >> b) & 1u) mbar_wait(bar0 + 8 * b, (owed_parity >> b) & 1u);
+    }
+    __syncthreads();
+  }
   if (wib == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(D::TMEM) : "memory");
 }
@@ -854,6 +888,7 @@ cudaError_t run_product(const LevelGeom& g, const DigitPlan& p, DigArgs a, cudaS
   a.w = p.w;
   a.sc = p.sc;
   a.err = p.err;
+  a.wait_ns = p.wait_ns;
   a.list = p.list;
   a.nlist = (int)p.nlist;
   a.list_blocks = DIM == 2 ? (int)((p.nlist + 63) / 64) : 0;  // 4 lanes a node
@@ -872,6 +907,8 @@ template <int DIM, int KIND>
 cudaError_t build_plan(const LevelGeom& g, const double* src, const unsigned char* nclass, const unsigned char* mask,
                        const int* prow, DigitPlan* p, unsigned char* tmp, int* rep, int* counts, cudaStream_t s) {
   using D = Dig<DIM, KIND>;
+  const char* env = getenv("FC_DIGIT_WAIT_NS");
+  p->wait_ns = env ? strtoull(env, nullptr, 10) : kWaitNs;
   const unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
   const int n = (int)g.nnodes, nb = (n + kListBlock - 1) / kListBlock;
   // rep[1], rep[2]: representatives; rep[4]: class nodes, rep[5]: classes

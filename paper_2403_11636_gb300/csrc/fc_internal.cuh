@@ -178,6 +178,7 @@ struct DigitPlan {
   double* w = nullptr;           // W, [class][slot][row]
   DigitScale* sc = nullptr;      // [class]
   unsigned* err = nullptr;       // the handle's error word
+  unsigned long long wait_ns = 0;  // after which a wait for products gives up
 };
 
 struct Level {
