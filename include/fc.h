@@ -436,7 +436,10 @@ const char* fc_batch_last_error(fc_batch b);
 fc_status fc_batch_destroy(fc_batch b);
 
 /* Wait for all work enqueued by the handle.  Errors: FC_ERR_INVALID (NULL
- * handle), FC_ERR_CUDA (the stream reported an error). */
+ * handle), FC_ERR_CUDA (the stream reported an error), FC_ERR_TIMEOUT (since
+ * the last fc_sync a kernel's wait for tensor-core products ran out: the
+ * results are complete, those products were formed in FP64, but the GPU was
+ * held up for a second; reported once). */
 fc_status fc_sync(fc_handle h);
 
 /* Message of the handle's last error ("" if none).  The string belongs to

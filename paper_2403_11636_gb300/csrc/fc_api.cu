@@ -1799,7 +1799,16 @@ fc_status fc_profile_read(fc_handle h, int kind, long long* launches, double* to
 
 fc_status fc_sync(fc_handle h) {
   if (!h) return FC_ERR_INVALID;
+  bool digits = false;
+  for (int l = 0; l < h->nlev && h->ready; ++l) digits = digits || h->lev[l].dig[0].on || h->lev[l].dig[1].on;
+  unsigned e = 0;
+  if (digits) CK(cudaMemcpyAsync(&e, h->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  if (e & kErrTimeout) {
+    CK(cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    return fail(h, FC_ERR_TIMEOUT, "a wait for tensor-core products ran out; the products were formed in FP64");
+  }
   return FC_OK;
 }
 

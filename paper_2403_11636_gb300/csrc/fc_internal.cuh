@@ -21,7 +21,9 @@ enum DevErr : unsigned {
   kErrSingularPatch = 2u,
   kErrSingularCoarse = 4u,
   kErrBadIndex = 8u,
-  kErrTimeout = 16u,  // a bounded wait gave up (fc_digits.cu; the products were formed in FP64)
+  // a bounded wait gave up (fc_digits.cu; the products were formed in FP64);
+  // fc_sync reports and clears it
+  kErrTimeout = 16u,
 };
 
 struct Shape {

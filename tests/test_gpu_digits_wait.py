@@ -40,3 +40,21 @@ def test_given_up_3d(fc, name, monkeypatch):
     x, b = inputs.uniform_array(s.ndof(), 5), inputs.uniform_array(s.ndof(), 7)
     want = s.smooth(x, b, nsweeps=2).cpu().numpy()
     assert rel(t.smooth(x, b, nsweeps=2).cpu().numpy() - x, want - x) <= 1e-11
+
+
+@pytest.mark.parametrize("name", ["384x352", "48"])
+def test_given_up_is_reported_once(fc, name, monkeypatch):
+    p = {**PROBS, **PROBS3}[name]
+    s = fc.Solver(p)
+    monkeypatch.setenv("FC_DIGIT_WAIT_NS", "0")
+    t = fc.Solver(p)
+    x, b = inputs.uniform_array(s.ndof(), 5), inputs.uniform_array(s.ndof(), 7)
+    t.sync()
+    s.smooth(x, b)
+    s.sync()
+    for _ in range(2):
+        t.smooth(x, b)
+        with pytest.raises(fc.FcError) as e:
+            t.sync()
+        assert e.value.code == fc.FC_ERR_TIMEOUT
+        t.sync()
