@@ -239,7 +239,11 @@ __device__ void fp64_product(const LevelGeom& g, const double* __restrict__ w, c
     const long long n = KIND == 0 ? pad_node(g, i0, i1, i2)
                                   : i0 + (long long)g.nn[0] * (i1 + (long long)(DIM == 3 ? g.nn[1] : 1) * i2);
     const double t = v[n * D::ND + c];
-    for (int q = 0; q < D::ND; ++q) y[q] = y[q] + w[(size_t)j * D::ND + q] * t;
+    for (int q = 0; q < D::ND; ++q) {
+      // (velocity components do not couple in the operator: 0 * infinity is no product)
+      if (KIND == 1 && c < DIM && q < DIM && q != c) continue;
+      y[q] = y[q] + w[(size_t)j * D::ND + q] * t;
+    }
   }
 }
 
