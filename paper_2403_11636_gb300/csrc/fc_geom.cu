@@ -1070,16 +1070,16 @@ __global__ void __launch_bounds__(32 << DIM)
                         &mlo, &mhi)) {
         if (mhi - mlo + 1 >= N) { mlo = 0; mhi = N - 1; }
       }
-      const int cnt = (int)(mhi - mlo + 1), n = (int)N;
-      const int start = (int)(((mlo % N) + N) % N);
+      // (64 bits: N passes 2^31 for radii of a million cells)
+      const long long cnt = mhi - mlo + 1, start = ((mlo % N) + N) % N;
       if (DIM == 2) {
-        for (int base = wib * 32; base < 2 * cnt; base += 32 * W) {
-          const int p = base + lane;
+        for (long long base = wib * 32; base < 2 * cnt; base += 32 * W) {
+          const long long p = base + lane;
           bool ok = false;
           double x[3] = {0.0, 0.0, 0.0}, nv[3] = {0.0, 0.0, 0.0}, w = 0.0;
           if (p < 2 * cnt) {
-            int m = start + p / 2;
-            if (m >= n) m -= n;
+            long long m = start + p / 2;
+            if (m >= N) m -= N;
             const double tt = dt * ((double)m + gq[p & 1]);
             const double ct = cos(tt), st = sin(tt);
             if (sh.type == 0) {
@@ -1104,24 +1104,25 @@ __global__ void __launch_bounds__(32 << DIM)
         // rings m0 .. m1 (two Gauss rings each) x the azimuth range, the
         // azimuths' cosines and sines tabulated kRing at a time
         const double w = r * r * (0.5 * dm) * dt;
-        const int nr = m1 >= m0 ? 2 * (int)(m1 - m0 + 1) : 0;
-        for (int q0 = 0; q0 < cnt; q0 += kRing) {
-          const int nq = cnt - q0 < kRing ? cnt - q0 : kRing;
+        const long long nr = m1 >= m0 ? 2 * (m1 - m0 + 1) : 0;
+        for (long long q0 = 0; q0 < cnt; q0 += kRing) {
+          const int nq = cnt - q0 < kRing ? (int)(cnt - q0) : kRing;
           __syncthreads();
           for (int q = tid; q < nq; q += 32 * W) {
-            int m = start + q0 + q;
-            if (m >= n) m -= n;
+            long long m = start + q0 + q;
+            if (m >= N) m -= N;
             const double ph = dt * ((double)m + 0.5);
             S.ct[q] = cos(ph);
             S.sn[q] = sin(ph);
           }
           __syncthreads();
-          for (int base = wib * 32; base < nr * nq; base += 32 * W) {
-            const int p = base + lane;
+          for (long long base = wib * 32; base < nr * nq; base += 32 * W) {
+            const long long p = base + lane;
             bool ok = false;
             double x[3] = {0.0, 0.0, 0.0}, nv[3] = {0.0, 0.0, 0.0};
             if (p < nr * nq) {
-              const int ring = p / nq, q = p - ring * nq;
+              const long long ring = p / nq;
+              const int q = (int)(p - ring * nq);
               const double mu = -1.0 + dm * ((double)(m0 + ring / 2) + gq[ring & 1]);
               const double st = sqrt(1.0 - mu * mu);
               const double ex = st * S.ct[q], ey = st * S.sn[q];
