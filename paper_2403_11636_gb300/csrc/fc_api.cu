@@ -418,7 +418,8 @@ void free_digit_plan(fc_handle h, DigitPlan* p) {
   dfree(h, p->cls);
   dfree(h, p->list);
   dfree(h, p->rows);
-  dfree(h, p->w);
+  dfree(h, p->wabs);
+  dfree(h, p->chk);
   dfree(h, p->sc);
   *p = DigitPlan();
 }
@@ -428,24 +429,26 @@ fc_status make_digit_plan(fc_handle h, Level& L, int kind, const double* src, co
   DigitPlan& p = L.dig[kind];
   const int part = kind == 0 ? 1 : 0;
   const size_t before = h->bytes[part];
-  unsigned char* tmp = nullptr;
-  int *rep = nullptr, *counts = nullptr;
-  char *rows = nullptr, *w = nullptr;
+  DigitScratch t;
+  char* rows = nullptr;
+  const size_t slots = (size_t)digit_plan_slots(G.dim, kind);
   CK(dalloc(h, &p.cls, (size_t)G.nnodes, part));
   CK(dalloc(h, &p.list, (size_t)G.nnodes, part));
   CK(dalloc(h, &rows, digit_plan_rows_bytes(G.dim, kind), part));
   p.rows = (uint4*)rows;
-  CK(dalloc(h, &w, digit_plan_w_bytes(G.dim, kind), part));
-  p.w = (double*)w;
-  CK(dalloc(h, &p.sc, 2, part));
-  CK(dalloc(h, &tmp, (size_t)G.nnodes, -1));
-  CK(dalloc(h, &rep, 6, -1));
-  CK(dalloc(h, &counts, (size_t)digit_plan_counts(G.nnodes), -1));
+  CK(dalloc(h, &p.wabs, slots, part));
+  CK(dalloc(h, &p.chk, slots, part));
+  CK(dalloc(h, &p.sc, 1, part));
+  CK(dalloc(h, &t.cls, (size_t)G.nnodes, -1));
+  CK(dalloc(h, &t.rep, 2, -1));
+  CK(dalloc(h, &t.counts, (size_t)digit_plan_counts(G.nnodes), -1));
+  CK(dalloc(h, &t.w, slots * G.nd, -1));
   p.err = h->d_err;
-  CK(build_digit_plan(G, kind, src, nclass, L.mask, L.prow, &p, tmp, rep, counts, h->stream));
-  dfree(h, tmp);
-  dfree(h, rep);
-  dfree(h, counts);
+  CK(build_digit_plan(G, kind, src, nclass, L.mask, L.prow, &p, t, h->stream));
+  dfree(h, t.cls);
+  dfree(h, t.rep);
+  dfree(h, t.counts);
+  dfree(h, t.w);
   p.on = G.nnodes - p.nlist >= G.nnodes / 16;
   if (!p.on) {
     free_digit_plan(h, &p);
@@ -944,7 +947,7 @@ size_t fc_footprint_estimate(const fc_grid* g, int depth, const fc_options* o) {
     const size_t dof = nodes * nd, pv = pad * nd;
     // class products: node classes, list of the other nodes, rows (two plans)
     for (int kind = 0; kind < (dim == 2 ? 2 : 1); ++kind)
-      held += nodes * 5 + 128 + digit_plan_rows_bytes(dim, kind) + digit_plan_w_bytes(dim, kind);
+      held += nodes * 5 + 128 + digit_plan_rows_bytes(dim, kind) + digit_plan_slots(dim, kind) * 18;
     if (l == 0) coarse_dof = dof;
     if (l == depth - 1) fine_dof = dof;
     held += nodes * nb * sp * 8 + nodes + dof * 8;                  // stencil, mask, Dirichlet values

@@ -153,34 +153,47 @@ struct AmrLevel {
   unsigned long long rows_flop = 0;  // 2 x (patch DoFs x free owned DoFs) summed over the patches
 };
 
-// Scales of a class's rows W as digits: |w| 2^(-delta on pressure columns) <
-// 2^rowexp; ok is zero where the class is empty or W is out of range.
+// Scales of the class rows W as digits: |w| 2^(-delta on pressure columns) <
+// 2^rowexp; floor as sum |w||v| has to be (fc_digits.cu); ok is zero where the
+// class is empty or W is out of range.
 struct DigitScale {
   int rowexp[4];
+  float floor[4];
   int delta;
   int ok;
 };
 
 // Levels of at least so many nodes get plans: below, a tile's fixed time (its
-// loads, digits and products follow one another) is more than the FP64 kernels
-// need.  GB300, us, class products / FP64 kernels: 2D patch apply 13 / 8 at
-// 65^2 nodes, 15 / 22 at 257^2, 27 / 80 at 1025 x 257, 164 / 790 at 1537^2; 2D
-// residual 13 / 5 at 65^2, 14 / 9 at 257^2, 20 / 29 at 1025 x 257, 125 / 263 at
-// 1537^2; 3D patch apply 172 + 417 (other patches) / 711 at 65^3 porous.
-constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 130000, kDigitApply3 = 100000;
+// loads, digits and products follow one another) and the CTAs that take their
+// nodes in FP64 are more than the FP64 kernels need.  GB300, us, class products /
+// FP64 kernels: 2D patch apply 13 / 8 at 65^2 nodes, 20 / 22 at 257^2, 33 / 50 at
+// 385^2, 32 / 80 at 1025 x 257, 272 / 790 at 1537^2; 2D residual of a random
+// vector 31 / 39 at 513^2, 22 / 39 at 1025 x 257, 164 / 263 at 1537^2, of a
+// solution (a small cross flow leaves the digits) 33 / 39 at 513^2, 43 / 39 at
+// 1025 x 257, 179 / 263 at 1537^2; 3D patch apply 172 + 417 (other patches) / 711 at 65^3 porous.
+constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 500000, kDigitApply3 = 100000;
 
 // Which nodes of a level take their product with the class rows on the tensor
 // cores, and those rows (fc_digits.cu).
 struct DigitPlan {
   bool on = false;
-  unsigned char* cls = nullptr;  // per node: bits 0-1 class of its product, bits 2-3 classes of products that read it
-  int* list = nullptr;           // nodes without a class, in order
+  unsigned char* cls = nullptr;  // per node: bit 0 class node, bit 1 a class node's product reads it
+  int* list = nullptr;           // the other nodes, in order
   long long nlist = 0;
-  uint4* rows = nullptr;         // W as a tensor-core operand, [class][step][1 KB]
-  double* w = nullptr;           // W, [class][slot][row]
-  DigitScale* sc = nullptr;      // [class]
+  uint4* rows = nullptr;         // W as a tensor-core operand
+  float4* wabs = nullptr;        // |W| by slot, largest first
+  unsigned short* chk = nullptr;  // those slots' offsets in a tile
+  DigitScale* sc = nullptr;
   unsigned* err = nullptr;       // the handle's error word
   unsigned long long wait_ns = 0;  // after which a wait for products gives up
+};
+
+// Scratch of a plan's construction
+struct DigitScratch {
+  unsigned char* cls = nullptr;  // nnodes
+  int* rep = nullptr;            // 2
+  int* counts = nullptr;         // digit_plan_counts
+  double* w = nullptr;           // digit_plan_slots * (dim + 1)
 };
 
 struct Level {
@@ -474,14 +487,14 @@ cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coe
                                const int* list = nullptr, long long nlist = 0);
 // FP64 class products on the tensor cores (fc_digits.cu).  kind 0: patch apply
 // (src = FP64 rows), 1: operator (src = stencil; 2D).  p's arrays are allocated by
-// the caller (sizes below); tmp nnodes bytes, rep 6 ints, counts
-// digit_plan_counts ints of scratch.  Synchronises.
+// the caller: cls and list by node, rows digit_plan_rows_bytes, wabs and
+// chk digit_plan_slots, one scale.  Synchronises.
 size_t digit_plan_rows_bytes(int dim, int kind);
-size_t digit_plan_w_bytes(int dim, int kind);
+int digit_plan_slots(int dim, int kind);
 int digit_plan_counts(long long nnodes);
 cudaError_t build_digit_plan(const LevelGeom& g, int kind, const double* src, const unsigned char* nclass,
-                             const unsigned char* mask, const int* prow, DigitPlan* p, unsigned char* tmp, int* rep,
-                             int* counts, cudaStream_t s);
+                             const unsigned char* mask, const int* prow, DigitPlan* p, const DigitScratch& t,
+                             cudaStream_t s);
 cudaError_t launch_digit_apply(const LevelGeom& g, const DigitPlan& p, const double* coef, const unsigned char* mask,
                                const double* rpad, double omega, double* x, const int* prow, cudaStream_t s);
 cudaError_t launch_digit_residual(const LevelGeom& g, const DigitPlan& p, const double* st, const unsigned char* mask,

@@ -3337,7 +3337,10 @@ cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coe
     const unsigned bl = (unsigned)((g.nnodes * t + 255) / 256);
     const unsigned nl = (unsigned)nlist;
     const double* c = (const double*)coef;
-    if (list) {
+    if (list && g.dim == 2) {
+      apply_fp64_kernel<2, 4, true>
+          <<<(unsigned)((nlist * 4 + 255) / 256), 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl);
+    } else if (list) {
       apply_fp64_kernel<3, 8, true>
           <<<(unsigned)((nlist * 8 + 255) / 256), 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl);
     } else if (g.dim == 2) {

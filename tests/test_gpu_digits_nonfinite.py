@@ -7,10 +7,11 @@ import pytest
 
 from paper_2403_11636_gb300 import inputs
 from tests.gpu_util import rel
-from tests.test_gpu_digits import OPER_TOL, PROBS, PROBS3
+from tests.test_gpu_digits import OPER_TOL, PROBS, PROBS3, square
 
 pytestmark = pytest.mark.gpu
-ALL = {**PROBS, **PROBS3}
+ALL = {**PROBS, **PROBS3,
+       "800x640": square(800, 640, nlevels=6), "open 800x640": square(800, 640, nlevels=6, preset=2)}
 
 
 @pytest.fixture(scope="module")
@@ -27,11 +28,11 @@ def around(p, at, r):
 
 
 # a fluid node away from obstacle and walls
-AT = {"384x352": (40, 300), "empty": (130, 100), "48": (4, 40, 6)}
+AT = {"384x352": (40, 300), "800x640": (80, 560), "open 800x640": (690, 90), "48": (4, 40, 6)}
 
 
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
-@pytest.mark.parametrize("name", ["384x352", "empty"])
+@pytest.mark.parametrize("name", ["800x640", "open 800x640"])
 def test_operator(fc, name, bad):
     p, nd = ALL[name], 3
     s = fc.Solver(p)

@@ -6,7 +6,7 @@ import pytest
 from oracle import oracle as O
 from paper_2403_11636_gb300 import inputs
 from tests.gpu_util import rel
-from tests.test_gpu_digits import OPER_TOL, PROBS, PROBS3, SWEEP_TOL, fields
+from tests.test_gpu_digits import OPER_TOL, PROBS, PROBS3, SWEEP_TOL, fields, square
 
 pytestmark = pytest.mark.gpu
 
@@ -17,7 +17,7 @@ def fc():
     return m
 
 
-# both classes in a tile, several tiles in both directions
+# several tiles in both directions, with an obstacle among them
 @pytest.mark.parametrize("name", ["384x352", "528x272"])
 def test_given_up_2d(fc, name, monkeypatch):
     monkeypatch.setenv("FC_DIGIT_WAIT_NS", "0")
@@ -29,6 +29,18 @@ def test_given_up_2d(fc, name, monkeypatch):
     assert rel(s.apply(x).cpu().numpy(), A @ x) <= OPER_TOL
     assert rel(s.residual(x, b).cpu().numpy(), b - A @ x) <= OPER_TOL
     assert rel(s.smooth(x, b).cpu().numpy() - x, L.sweep(b, x) - x) <= SWEEP_TOL
+
+
+def test_given_up_operator(fc, monkeypatch):
+    p = square(800, 640, nlevels=6)
+    s = fc.Solver(p)
+    monkeypatch.setenv("FC_DIGIT_WAIT_NS", "0")
+    t = fc.Solver(p)
+    x, b = inputs.uniform_array(s.ndof(), 5), s.rhs()
+    assert rel(t.apply(x).cpu().numpy(), s.apply(x).cpu().numpy()) <= OPER_TOL
+    assert rel(t.residual(x, b).cpu().numpy(), s.residual(x, b).cpu().numpy()) <= OPER_TOL
+    with pytest.raises(fc.FcError):
+        t.sync()
 
 
 @pytest.mark.parametrize("name", ["48", "pores"])
