@@ -3341,8 +3341,13 @@ cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coe
       apply_fp64_kernel<2, 4, true>
           <<<(unsigned)((nlist * 4 + 255) / 256), 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl);
     } else if (list) {
-      apply_fp64_kernel<3, 8, true>
-          <<<(unsigned)((nlist * 8 + 255) / 256), 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl);
+      const unsigned lb = (unsigned)((nlist * t + 255) / 256);
+      switch (t) {
+        case 4: apply_fp64_kernel<3, 4, true><<<lb, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl); break;
+        case 16: apply_fp64_kernel<3, 16, true><<<lb, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl); break;
+        case 32: apply_fp64_kernel<3, 32, true><<<lb, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl); break;
+        default: apply_fp64_kernel<3, 8, true><<<lb, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, list, nl); break;
+      }
     } else if (g.dim == 2) {
       apply_fp64_kernel<2, 4, false><<<bl, 256, 0, s>>>(g, c, mask, rpad, omega, x, prow, nullptr, 0);
     } else {
