@@ -440,7 +440,7 @@ fc_status make_digit_plan(fc_handle h, Level& L, int kind, const double* src, co
   CK(dalloc(h, &p.chk, slots, part));
   CK(dalloc(h, &p.sc, 1, part));
   CK(dalloc(h, &t.cls, (size_t)G.nnodes, -1));
-  CK(dalloc(h, &t.rep, 2, -1));
+  CK(dalloc(h, &t.rep, 3, -1));
   CK(dalloc(h, &t.counts, (size_t)digit_plan_counts(G.nnodes), -1));
   CK(dalloc(h, &t.w, slots * G.nd, -1));
   p.err = h->d_err;
@@ -449,7 +449,6 @@ fc_status make_digit_plan(fc_handle h, Level& L, int kind, const double* src, co
   dfree(h, t.rep);
   dfree(h, t.counts);
   dfree(h, t.w);
-  p.on = G.nnodes - p.nlist >= G.nnodes / 16;
   if (!p.on) {
     free_digit_plan(h, &p);
     h->bytes[part] = before;

@@ -84,7 +84,7 @@ struct Dig {
   // that some row of a block can read
   static constexpr int FAR = 2 * R * (1 + HX + (DIM == 3 ? HX * HY : 0));
   static constexpr int PLANE = NBLK * 128 + FAR + 8;
-  static constexpr int THREADS = 256;
+  static constexpr int THREADS = 256, PER_SM = DIM == 3 ? 1 : 3;  // CTAs an SM, by shared memory
   // W is read in pieces of CS steps, NST pieces in flight
   static constexpr int CS = DIM == 3 ? 12 : STEPS, NST = DIM == 3 ? 3 : 1, NCH = (STEPS + CS - 1) / CS;
   static constexpr int STEPB = 2 * N * 16;  // bytes of W a step
@@ -333,7 +333,7 @@ constexpr int kFloor = -10;
 // next tile's values loaded during the products, were slower: 196 against 164
 // us for the 1537^2 patch apply.)
 template <int DIM, int KIND>
-__global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, DIM == 3 ? 1 : 3)
+__global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, Dig<DIM, KIND>::PER_SM)
     digit_product_kernel(LevelGeom g, DigArgs a, int tiles_x, int tiles_y) {
   using D = Dig<DIM, KIND>;
   constexpr int ND = D::ND, R = D::R;
@@ -827,6 +827,23 @@ __global__ void digit_tag_kernel(LevelGeom g, const unsigned char* __restrict__ 
   if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, n);
 }
 
+// counts the tiles that hold class nodes (a CTA each)
+template <int DIM, int KIND>
+__global__ void __launch_bounds__(128) digit_tiles_kernel(LevelGeom g, const unsigned char* __restrict__ cls, int tiles_x,
+                                                          int tiles_y, int* __restrict__ count) {
+  using D = Dig<DIM, KIND>;
+  const int tq = blockIdx.x / tiles_x;
+  const int b0 = blockIdx.x % tiles_x * D::TX + D::R, b1 = (DIM == 3 ? tq % tiles_y : tq) * D::TY + D::R;
+  const int b2 = DIM == 3 ? tq / tiles_y * D::TZ + D::R : 0;
+  bool any = false;
+  for (int t = threadIdx.x; t < D::TX * D::TY * D::TZ; t += blockDim.x) {
+    const int i = b0 + t % D::TX, j = b1 + t / D::TX % D::TY, k = b2 + t / (D::TX * D::TY);
+    if (i < g.nn[0] && j < g.nn[1] && (DIM == 2 || k < g.nn[2]))
+      any = any || (cls[i + (long long)g.nn[0] * (j + (long long)(DIM == 3 ? g.nn[1] : 1) * k)] & 1);
+  }
+  if (__syncthreads_or(any) && threadIdx.x == 0) atomicAdd(count, 1);
+}
+
 // the nodes without a class, in order
 constexpr int kListBlock = 1024;
 __global__ void digit_list_count_kernel(int n, const unsigned char* __restrict__ cls, int* __restrict__ counts) {
@@ -1005,6 +1022,24 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+template <int DIM, int KIND>
+void tiles_of(const LevelGeom& g, int* tx, int* ty, int* tz) {
+  using D = Dig<DIM, KIND>;
+  *tx = (g.nn[0] - 2 * D::R + D::TX - 1) / D::TX;
+  *ty = (g.nn[1] - 2 * D::R + D::TY - 1) / D::TY;
+  *tz = DIM == 3 ? (g.nn[2] - 2 * D::R + D::TZ - 1) / D::TZ : 1;
+}
+
+// Class nodes that a wave of tiles (one on every place of the GPU) has to take
+// off the FP64 kernels to pay for its time.  GB300, measured where both sides
+// are equal: 3D apply 16,300 to 18,500 a wave at 49^3, 57^3, 65^3, 73^3 and 81^3
+// nodes with 0 to 100 spheres (49^3, 318 us in FP64: 0 spheres, 79,500 class
+// nodes, 212; 12, 61,500, 251; 40, 26,000, 346.  65^3, 715 us: 0, 205,000, 364;
+// 40, 102,000, 605; 100, 43,000, 753); 2D apply 37,000 and 2D operator 89,000 by
+// the times of grids without obstacles (a wave 15 and 10 us).
+template <int DIM, int KIND>
+constexpr long long kPerWave = DIM == 3 ? 18500 : KIND == 0 ? 40000 : 100000;
+
 // The plan's list in FP64.  A short one is taken by the first CTAs of the same
 // launch (a launch less).  A long one has a launch of its own: beside tiles,
 // whose shared memory leaves 24 warps an SM, it is bound by latency (326,000
@@ -1048,10 +1083,9 @@ cudaError_t run_product(const LevelGeom& g, const DigitPlan& p, DigArgs a, cudaS
   auto kern = digit_product_kernel<DIM, KIND>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D::BYTES);
   if (e != cudaSuccess) return e;
-  const int tx = (g.nn[0] - 2 * D::R + D::TX - 1) / D::TX, ty = (g.nn[1] - 2 * D::R + D::TY - 1) / D::TY;
-  const int tz = DIM == 3 ? (g.nn[2] - 2 * D::R + D::TZ - 1) / D::TZ : 1;
-  const unsigned blocks = (unsigned)a.list_blocks + (unsigned)tx * ty * tz;
-  kern<<<blocks, D::THREADS, D::BYTES, s>>>(g, a, tx, ty);
+  int tx, ty, tz;
+  tiles_of<DIM, KIND>(g, &tx, &ty, &tz);
+  kern<<<(unsigned)a.list_blocks + (unsigned)tx * ty * tz, D::THREADS, D::BYTES, s>>>(g, a, tx, ty);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -1059,27 +1093,36 @@ cudaError_t run_product(const LevelGeom& g, const DigitPlan& p, DigArgs a, cudaS
 template <int DIM, int KIND>
 cudaError_t build_plan(const LevelGeom& g, const double* src, const unsigned char* nclass, const unsigned char* mask,
                        const int* prow, DigitPlan* p, const DigitScratch& t, cudaStream_t s) {
+  using D = Dig<DIM, KIND>;
   const char* env = getenv("FC_DIGIT_WAIT_NS");
   p->wait_ns = env ? strtoull(env, nullptr, 10) : kWaitNs;
   const unsigned blocks = (unsigned)((g.nnodes + 255) / 256);
   const int n = (int)g.nnodes, nb = (n + kListBlock - 1) / kListBlock;
-  const int init[2] = {0x7fffffff, 0};  // representative, class nodes
+  const int init[3] = {0x7fffffff, 0, 0};  // representative, class nodes, tiles with some
   cudaError_t e = cudaMemcpyAsync(t.rep, init, sizeof(init), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   digit_class_kernel<DIM, KIND><<<blocks, 256, 0, s>>>(g, nclass, mask, t.cls, t.rep);
   if (KIND == 1) digit_compare_kernel<DIM><<<blocks, 256, 0, s>>>(g, src, t.cls, t.rep);
   digit_tag_kernel<DIM, KIND><<<blocks, 256, 0, s>>>(g, t.cls, p->cls, t.rep + 1);
+  int tx, ty, tz;
+  tiles_of<DIM, KIND>(g, &tx, &ty, &tz);
+  if (tx > 0 && ty > 0 && tz > 0)
+    digit_tiles_kernel<DIM, KIND><<<(unsigned)tx * ty * tz, 128, 0, s>>>(g, p->cls, tx, ty, t.rep + 2);
   digit_list_count_kernel<<<nb, kListBlock, 0, s>>>(n, p->cls, t.counts);
   digit_list_scan_kernel<<<1, 1024, 0, s>>>(nb, t.counts);
   digit_list_place_kernel<<<nb, kListBlock, 0, s>>>(n, p->cls, t.counts, p->list);
   digit_rows_kernel<DIM, KIND><<<1, 256, 0, s>>>(g, src, prow, t.rep, t.w, p->rows, p->wabs, p->chk, p->sc);
-  note_launches(6 + KIND);
+  note_launches(7 + KIND);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  int got = 0;
-  e = cudaMemcpyAsync(&got, t.rep + 1, sizeof(got), cudaMemcpyDeviceToHost, s);
+  int got[2] = {0, 0}, dev = 0, nsm = 0;
+  e = cudaMemcpyAsync(got, t.rep + 1, sizeof(got), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  p->nlist = g.nnodes - got;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  p->nlist = g.nnodes - got[0];
+  const long long places = std::max(1, D::PER_SM * nsm);
+  p->on = got[0] > 0 && got[0] >= kPerWave<DIM, KIND> * ((got[1] + places - 1) / places);
   return e;
 }
 

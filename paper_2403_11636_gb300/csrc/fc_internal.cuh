@@ -163,14 +163,14 @@ struct DigitScale {
   int ok;
 };
 
-// Levels of at least so many nodes get plans: below, a tile's fixed time (its
-// loads, digits and products follow one another) and the CTAs that take their
-// nodes in FP64 are more than the FP64 kernels need.  GB300, us, class products /
-// FP64 kernels: 2D patch apply 13 / 8 at 65^2 nodes, 20 / 22 at 257^2, 33 / 50 at
-// 385^2, 32 / 80 at 1025 x 257, 272 / 790 at 1537^2; 2D residual of a random
-// vector 31 / 39 at 513^2, 22 / 39 at 1025 x 257, 164 / 263 at 1537^2, of a
-// solution (a small cross flow leaves the digits) 33 / 39 at 513^2, 43 / 39 at
-// 1025 x 257, 179 / 263 at 1537^2; 3D patch apply 172 + 417 (other patches) / 711 at 65^3 porous.
+// Levels of at least so many nodes can get plans (fc_digits.cu decides by their
+// class nodes): below, a tile's fixed time (its loads, digits and products
+// follow one another) and the CTAs that take their nodes in FP64 are more than
+// the FP64 kernels need.  GB300, us, class products / FP64 kernels: 2D patch apply
+// 13 / 8 at 65^2 nodes, 20 / 22 at 257^2, 33 / 50 at 385^2, 32 / 80 at 1025 x 257,
+// 272 / 790 at 1537^2; 2D residual of a random vector 31 / 39 at 513^2, 22 / 39 at
+// 1025 x 257, 164 / 263 at 1537^2, of a solution (a small cross flow leaves the
+// digits) 33 / 39 at 513^2, 43 / 39 at 1025 x 257, 179 / 263 at 1537^2.
 constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 500000, kDigitApply3 = 100000;
 
 // Which nodes of a level take their product with the class rows on the tensor
@@ -191,7 +191,7 @@ struct DigitPlan {
 // Scratch of a plan's construction
 struct DigitScratch {
   unsigned char* cls = nullptr;  // nnodes
-  int* rep = nullptr;            // 2
+  int* rep = nullptr;            // 3
   int* counts = nullptr;         // digit_plan_counts
   double* w = nullptr;           // digit_plan_slots * (dim + 1)
 };
@@ -488,7 +488,7 @@ cudaError_t launch_patch_apply(const LevelGeom& g, fc_prec prec, const void* coe
 // FP64 class products on the tensor cores (fc_digits.cu).  kind 0: patch apply
 // (src = FP64 rows), 1: operator (src = stencil; 2D).  p's arrays are allocated by
 // the caller: cls and list by node, rows digit_plan_rows_bytes, wabs and
-// chk digit_plan_slots, one scale.  Synchronises.
+// chk digit_plan_slots, one scale.  Sets p->on where the plan pays.  Synchronises.
 size_t digit_plan_rows_bytes(int dim, int kind);
 int digit_plan_slots(int dim, int kind);
 int digit_plan_counts(long long nnodes);
