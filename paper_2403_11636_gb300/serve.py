@@ -202,10 +202,13 @@ class BatchServer:
     joined), new requests joining and converged ones (or ones past
     ``max_iters`` iterations) leaving between cycles; a request's result
     holds ``final_fn(state)`` of its last cycle as its solution.  ``join_s``:
-    how long an idle live driver that has one request ready waits for a second
-    whose setup is running (two requests cost a cycle little more than one;
-    setups of 20 ms, as short as the gaps between requests, would otherwise
-    never meet in a batch)."""
+    how long an idle live driver that has one request ready may wait for a
+    second whose setup is running, so that the two share their cycles; 0: not
+    at all, the lowest latency of a single request.  It waits only for a
+    setup expected to end in that time: one as long as the ready request's,
+    times the ratio of their footprints where that is larger.  (16^3 porous
+    requests 20 ms apart, each 33 to 35 ms from arrival to result alone: with 30
+    ms, pairs of 53 and 33.)"""
 
     def __init__(self, setup_fn: Callable, round_fn: Callable, release_fn: Callable, footprint_fn: Callable,
                  budget_bytes: float, slots: int, max_batch: int = 64, make_stream: Callable = lambda: None,
@@ -231,11 +234,13 @@ class BatchServer:
     @classmethod
     def gpu(cls, budget_bytes: float = 150e9, slots: int = 8, prec: str = "fp32", dedup: int = 1,
             tc: str = "none", tile=(16, 256, 8), keep_solutions: bool = False, rtol: Optional[float] = None,
-            max_batch: int = 64, gather_s: float = 0.0, live: bool = False, cycle_iters: int = 30):
+            max_batch: int = 64, gather_s: float = 0.0, live: bool = False, cycle_iters: int = 30,
+            join_s: float = 0.03):
         """libfc form.  ``live``: one FGMRES restart cycle of ``cycle_iters``
         iterations (the solvers' restart length) per batched call, requests
         joining and leaving between cycles; the batch is rebuilt only when
-        its membership changes."""
+        its membership changes.  ``join_s`` (see the class) concerns live
+        serving."""
         import torch
         from . import fc
 
@@ -291,7 +296,7 @@ class BatchServer:
 
         return cls(setup, solve_round, release, footprint, budget_bytes, slots, max_batch,
                    make_stream=lambda: torch.cuda.Stream(), gather_s=gather_s,
-                   cycle_fn=solve_cycle if live else None, final_fn=final, join_s=0.03)
+                   cycle_fn=solve_cycle if live else None, final_fn=final, join_s=join_s)
 
     def run(self, requests: List[Request]) -> List[BatchResult]:
         """Serve ``requests`` (arrival times relative to the call) to completion."""
@@ -301,7 +306,7 @@ class BatchServer:
                 raise ValueError(f"request {r.rid} needs more than the whole budget")
         lock = threading.Condition()
         st = {"used": 0.0, "free_slots": list(range(self.slots)), "ready": [], "results": [], "errors": [],
-              "setting_up": 0, "solving": 0, "done_admitting": False, "rounds": 0}
+              "setting_up": 0, "solving": 0, "done_admitting": False, "rounds": 0, "running": {}}
         streams = [self.make_stream() for _ in range(self.slots)]
         driver_stream = self.make_stream()
         t0 = self.clock()
@@ -319,11 +324,13 @@ class BatchServer:
                 with lock:
                     st["ready"].append((req, h, slot, fp, admitted, ts))
                     st["setting_up"] -= 1
+                    del st["running"][slot]
                     lock.notify_all()
             except Exception as e:  # a failed setup is reported; its slot is freed
                 with lock:
                     st["errors"].append((req.rid, repr(e)))
                     st["setting_up"] -= 1
+                    st["running"].pop(slot, None)
                     finish(slot, fp)
                     lock.notify_all()
 
@@ -364,6 +371,11 @@ class BatchServer:
                         finish(slot, fp)
                         lock.notify_all()
 
+        def joins_by(deadline):
+            # a setup is expected to end in time for the one ready request
+            _, _, _, fp, _, ts = st["ready"][0]
+            return any(t + ts * max(1.0, f / fp if fp > 0 else 1.0) <= deadline for t, f in st["running"].values())
+
         def live_driver():
             active = []  # requests in flight: [req, h, slot, fp, admitted, ts, state, iterations, joined, first]
             while True:
@@ -371,8 +383,8 @@ class BatchServer:
                     while not st["ready"] and not active and not (st["done_admitting"] and st["setting_up"] == 0):
                         lock.wait(timeout=0.05)
                     deadline = self.clock() + self.join_s
-                    while (not active and st["setting_up"] > 0 and len(st["ready"]) == 1 and self.max_batch > 1
-                           and self.clock() < deadline):
+                    while (not active and len(st["ready"]) == 1 and self.max_batch > 1 and self.clock() < deadline
+                           and joins_by(deadline)):
                         lock.wait(timeout=min(0.01, max(0.0, deadline - self.clock())))
                     room = self.max_batch - len(active)
                     joining = st["ready"][:room]
@@ -433,6 +445,7 @@ class BatchServer:
                     slot = st["free_slots"].pop()
                     st["used"] += fp
                     st["setting_up"] += 1
+                    st["running"][slot] = (self.clock(), fp)
                     th = threading.Thread(target=setup_worker, args=(slot, req, fp, now), daemon=True)
                     threads.append(th)
                     th.start()
