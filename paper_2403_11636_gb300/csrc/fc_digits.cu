@@ -1117,12 +1117,15 @@ cudaError_t build_plan(const LevelGeom& g, const double* src, const unsigned cha
   if (e != cudaSuccess) return e;
   int got[2] = {0, 0}, dev = 0, nsm = 0;
   e = cudaMemcpyAsync(got, t.rep + 1, sizeof(got), cudaMemcpyDeviceToHost, s);
+  DigitScale sc;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&sc, p->sc, sizeof(sc), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   p->nlist = g.nnodes - got[0];
   const long long places = std::max(1, D::PER_SM * nsm);
-  p->on = got[0] > 0 && got[0] >= kPerWave<DIM, KIND> * ((got[1] + places - 1) / places);
+  p->on = sc.ok && got[0] > 0 && got[0] >= kPerWave<DIM, KIND> * ((got[1] + places - 1) / places);
   return e;
 }
 
