@@ -745,7 +745,18 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, Dig<DIM, KIND>::PER_S
   const int nleft = snleft;
   if (nleft == 0) return;
   int* soff = reinterpret_cast<int*>(smem + D::O_ROWS);
-  if (KIND == 0) slot_table<DIM>(g, soff);
+  if constexpr (KIND == 0) {
+    slot_table<DIM>(g, soff);
+  } else if (nleft >= D::THREADS / 2) {
+    // many: a thread each (1025 x 257 nodes at the solution, 10,000 nodes in few
+    // tiles: 43 -> 34 us a launch)
+    for (int t = tid; t < nleft; t += D::THREADS) {
+      const int m = sleft[t];
+      residual_node<DIM, 0, 1>(g, a.coef, a.mask, a.v, a.b, a.r, a.rpad, nullptr,
+                               bx + m % D::HX + g.nn[0] * (by + m / D::HX), true);
+    }
+    return;
+  }
   for (int base = 0; base < nleft; base += D::THREADS / TPP) {
     const int gi = base + tid / TPP;
     const bool valid = gi < nleft;

@@ -168,10 +168,11 @@ struct DigitScale {
 // follow one another) and the CTAs that take their nodes in FP64 are more than
 // the FP64 kernels need.  GB300, us, class products / FP64 kernels: 2D patch apply
 // 13 / 8 at 65^2 nodes, 20 / 22 at 257^2, 33 / 50 at 385^2, 32 / 80 at 1025 x 257,
-// 272 / 790 at 1537^2; 2D residual of a random vector 31 / 39 at 513^2, 22 / 39 at
-// 1025 x 257, 164 / 263 at 1537^2, of a solution (a small cross flow leaves the
-// digits) 33 / 39 at 513^2, 43 / 39 at 1025 x 257, 179 / 263 at 1537^2.
-constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 500000, kDigitApply3 = 100000;
+// 272 / 790 at 1537^2; 2D residual of a random vector 21 / 21 at 385^2, 31 / 39 at
+// 513^2, 22 / 39 at 1025 x 257, 164 / 263 at 1537^2, of a solution (a small cross
+// flow leaves the digits) 31 / 39 at 513^2, 34 / 39 at 1025 x 257, 174 / 263 at
+// 1537^2.
+constexpr long long kDigitApply2 = 50000, kDigitResidual2 = 130000, kDigitApply3 = 100000;
 
 // Which nodes of a level take their product with the class rows on the tensor
 // cores, and those rows (fc_digits.cu).

@@ -19,7 +19,7 @@ from paper_2403_11636_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 EMPTY2 = dataclasses.replace(inputs.channel_2d(0, n=64, nlevels=5), n=(384, 368), shapes=np.zeros((0, 9)), omega=1.0)
-LARGE2 = dataclasses.replace(EMPTY2, n=(768, 672), nlevels=6)   # operator: from 500,000 nodes
+LARGE2 = dataclasses.replace(EMPTY2, n=(768, 672), nlevels=6)   # operator
 EMPTY3 = dataclasses.replace(inputs.porous_3d(0, n=8, nspheres=1, nlevels=4), n=(48, 56, 48), shapes=np.zeros((0, 9)),
                              omega=1.0)
 KINDS = ["plain", "ramp", "spikes", "exponents", "components"]

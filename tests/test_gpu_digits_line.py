@@ -55,7 +55,7 @@ def test_line_3d(fc, n, nlevels, spheres, launches):
 
 
 @pytest.mark.parametrize("n, nlevels, radius, apply, operator", [
-    (192, 6, 0.2, False, False), (256, 6, 0.2, True, False), (256, 6, 0.35, False, False), (512, 7, 0.2, True, False),
+    (192, 6, 0.2, False, False), (256, 6, 0.2, True, False), (256, 6, 0.35, False, False), (384, 6, 0.2, True, True), (512, 7, 0.2, True, True),
     (1024, 8, 0.2, True, True), (1024, 8, 0.48, True, True)])
 def test_line_2d(fc, n, nlevels, radius, apply, operator, monkeypatch):
     """(A patch apply meets the right-hand side of x = 0, smoothed once.)"""
