@@ -39,8 +39,8 @@
 // rounding of the values, at most 2^(E-63) sum|w| (the antidiagonals that are
 // left out and W's own rounding are 2^-66 of max|w| max|v|).  That is relative to
 // the tile's largest value, not to what a node reads, so each node's sum |w||v|
-// is formed beside it in float32, and a node where it is below 2^(E-10) sum|w|
-// for some row leaves the digits: a result's error is at most about 2^-53
+// is formed beside it in float32, and a node where it is below 2^(E-11) sum|w|
+// for some row leaves the digits: a result's error is at most about 2^-52
 // sum |w||v|, where a chain of FP64 fused multiply-adds has that for every
 // partial sum (measured: see kFloor).  The nodes
 // that leave, and all of a tile that holds an infinity or NaN, whose exponent is
@@ -56,6 +56,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fc_node.cuh"
 
@@ -320,13 +321,15 @@ __device__ __forceinline__ void store_product(const LevelGeom& g, const DigArgs&
 }
 
 // A node takes its digits' result where sum |w||v| >= 2^kFloor 2^E sum|w| in every
-// row: the values' rounding is then at most 2^-53 sum |w||v|.  Error in 2^-53 sum
-// |w||v|, root mean square (largest), here / the FP64 kernels: random values,
-// patch apply 2D 0.11 (0.6) / 0.31 (1.7), 3D 0.08 (0.4) / 0.38 (2.5), operator
-// 0.18 (0.9) / 0.55 (3.5); a ramp of 1.5 bits a column 0.34 (2.0) / 0.36 (1.9),
-// 0.28 (1.5) / 0.32 (1.6), 0.41 (2.4) / 0.59 (4.2); spikes of 2^40 0.29 (3.3) /
-// 0.39 (3.5), 0.69 (7.4) / 0.81 (8.1), 0.35 (2.3) / 0.56 (5.4).
-constexpr int kFloor = -10;
+// row: the values' rounding is then at most 2^-52 sum |w||v|, and at random below
+// that of the FP64 sums.  Error in 2^-53 sum |w||v|, root mean square (largest), of
+// nodes that read random values 2^-k times those of a few others in the tile,
+// all by digits / by the FP64 kernels: patch apply 2D k = 4 0.11 (0.6) / 0.31
+// (1.7), k = 10 0.11 (0.6), k = 11 0.57 (2.7), k = 14 3.7; 3D k = 4 0.08 (0.4) /
+// 0.38 (2.2), k = 9 0.15, k = 10 0.25 (1.5), k = 11 0.65 (4.1); operator k = 4 0.18
+// (0.9) / 0.55 (3.4), k = 9 0.30, k = 10 0.47 (3.2), k = 11 1.2 (9.6).  Random
+// values have half their bound in the mean, so -11 is k = 10.
+constexpr int kFloor = -11;
 
 // 2D: the first list_blocks CTAs take the nodes of the plan's list in FP64.
 // The others take a tile each.  (CTAs that keep W and walk over the tiles, the
@@ -757,18 +760,24 @@ __global__ void __launch_bounds__(Dig<DIM, KIND>::THREADS, Dig<DIM, KIND>::PER_S
     }
     return;
   }
-  for (int base = 0; base < nleft; base += D::THREADS / TPP) {
-    const int gi = base + tid / TPP;
-    const bool valid = gi < nleft;
-    const int m = sleft[valid ? gi : nleft - 1];
-    const int i = bx + m % D::HX, j = by + (DIM == 3 ? (m / D::HX) % D::HY : m / D::HX);
-    const int k = DIM == 3 ? bz + m / (D::HX * D::HY) : 0;
-    const int node = i + g.nn[0] * (j + (DIM == 3 ? g.nn[1] : 1) * k);
-    if constexpr (KIND == 0)
-      apply_fp64_patch<DIM, TPP>(g, a.coef, a.mask, a.v, a.omega, a.x, a.prow, soff, (unsigned)node, valid);
-    else
-      residual_node<DIM, 0, TPP>(g, a.coef, a.mask, a.v, a.b, a.r, a.rpad, nullptr, node, valid);
-  }
+  auto by_lanes = [&](auto lanes) {
+    constexpr int L = decltype(lanes)::value;
+    for (int base = 0; base < nleft; base += D::THREADS / L) {
+      const int gi = base + tid / L;
+      const bool valid = gi < nleft;
+      const int m = sleft[valid ? gi : nleft - 1];
+      const int i = bx + m % D::HX, j = by + (DIM == 3 ? (m / D::HX) % D::HY : m / D::HX);
+      const int k = DIM == 3 ? bz + m / (D::HX * D::HY) : 0;
+      const int node = i + g.nn[0] * (j + (DIM == 3 ? g.nn[1] : 1) * k);
+      if constexpr (KIND == 0)
+        apply_fp64_patch<DIM, L>(g, a.coef, a.mask, a.v, a.omega, a.x, a.prow, soff, (unsigned)node, valid);
+      else
+        residual_node<DIM, 0, L>(g, a.coef, a.mask, a.v, a.b, a.r, a.rpad, nullptr, node, valid);
+    }
+  };
+  // (3D: 3.6 us for 8 nodes at a warp each, 13 us for 32 at 8 lanes)
+  if (DIM == 3 && nleft <= 24) by_lanes(std::integral_constant<int, 32>());
+  else by_lanes(std::integral_constant<int, TPP>());
 }
 
 // ---- plan ------------------------------------------------------------------
