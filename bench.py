@@ -17,7 +17,7 @@ of profiled solves after the timed ones.  With FP64 rows the patch apply is
 bound by the FP64 pipe (GB300 runs FP64 at 1/64 of the FP32 rate), so its
 roofline is FP64 FLOP/s against the nominal pipe peak, with the live FMA
 probe and the HBM fraction beside it.  The operations counted are those of
-the FP64 pipe; uncut patches take the tensor cores (fc_digits.cu).
+the FP64 pipe; uncut fluid patches take the tensor cores (fc_digits.cu).
 
 --impl reference times the FP64 CPU oracle (the plain implementation the
 tests compare against) on the host cores, on a bounded sample of the same
@@ -324,8 +324,8 @@ def run_ours(args, rank, world, local_rank):
     hbm, peak_kind = peaks()
     avg_fine_ms = ms_fine / max(n_fine, 1)
     gbs = bytes_fine / (avg_fine_ms * 1e-3) / 1e9 if ms_fine > 0 else 0.0
-    # the FP64 pipe's share: uncut patches of large levels are multiplied on
-    # the tensor cores (exact digit products) in the same launches
+    # the FP64 pipe's share: uncut fluid patches of large levels are multiplied
+    # on the tensor cores (exact digit products) in the same launches
     tflops = flops_pipe / (avg_fine_ms * 1e-3) / 1e12 if ms_fine > 0 else 0.0
     traffic = load_traffic(args.prec) if not args.dedup else None
     if args.prec == "fp64":
@@ -353,7 +353,7 @@ def run_ours(args, rank, world, local_rank):
                                "r~U[0.04,0.12], alpha 1e-8, octree depth 3, 5 levels, V(2,2), "
                                "FGMRES(30) rtol 1e-8, Q1-Q1 (1,098,500 DoFs)",
                    "cache": args.cache, "patch_rows": args.prec, "shared_class_blocks": bool(args.dedup),
-                   "l2": "inputs larger than L2 (cached rows 4.1 GB per V-cycle)",
+                   "l2": f"inputs larger than L2 (a finest-level patch apply reads {bytes_fine / 1e9:.1f} GB)",
                    "iterations": its_list[0], "relres": max(rr_list), "setup_ms": setup_ms,
                    "solves_per_s": world * args.steps / (total_ms * 1e-3),
                    "latency_ms": {"p50": pct(step_ms, 50), "p99": pct(step_ms, 99), "n": len(step_ms),
@@ -1149,7 +1149,7 @@ def load_traffic(prec):
     """DRAM bytes per finest-level launch of the patch apply, from the
     committed ncu summary of this precision (a line 'traffic_bytes_64: N')."""
     path = os.path.join(ROOT, "profiles", f"patch_apply_{prec}_porous48.md")
-    # the summary is of the per-patch layout (one stored block per patch)
+    # the summary is of the layout with a stored block for every patch
     try:
         for line in open(path):
             if line.strip().startswith("traffic_bytes_64:"):

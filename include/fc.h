@@ -131,7 +131,9 @@ typedef struct {
   double force[3];
   int dedup;           /* 1: patches with bit-identical blocks L_i (uncut, one alpha, away
                           from constraints) share one stored row/factor block; 0: one block
-                          per patch (the paper's layout).  Same results either way. */
+                          per patch (the paper's layout; the tensor-core products of
+                          uncut fluid patches on large FP64 levels read one of them in
+                          either case).  Same results either way. */
   int tc;              /* float32 / bfloat16 rows with dedup 1: how the V-cycle applies the
                           shared class blocks.  0: CUDA cores (float32 FMA); 1: tensor cores,
                           rows and residual rounded to TF32; 2: tensor cores, rows and residual
@@ -325,8 +327,8 @@ size_t fc_footprint_estimate(const fc_grid* g, int depth, const fc_options* o);
  * kind: 0 patch apply (all levels), 1 residual (smoother), 2 V-cycle,
  * 3 patch-cache build, 4 patch apply on the finest level only, 5 the same
  * launches with FP64 rows, bytes_per_launch being the operations that they
- * leave to the FP64 pipe (uncut patches of large levels take the tensor
- * cores).
+ * leave to the FP64 pipe (uncut fluid patches of large levels take the tensor
+ * cores; those that leave the digits for their accuracy are not counted).
  * Reading synchronises and resets the counters of that kind. */
 fc_status fc_profile_enable(fc_handle h, int on);
 fc_status fc_profile_read(fc_handle h, int kind, long long* launches, double* total_ms,

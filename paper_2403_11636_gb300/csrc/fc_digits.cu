@@ -37,15 +37,15 @@
 // not used); those of d >= 6, of weight 2^-48 and less, could in 3D round by a
 // unit if nearly all digits were largest and of one sign.  What is lost is the
 // rounding of the values, at most 2^(E-63) sum|w| (the antidiagonals that are
-// left out and W's own rounding are 2^-66 of max|w| max|v|).  That is relative to
-// the tile's largest value, not to what a node reads, so each node's sum |w||v|
+// left out and W's own rounding are 2^-66 of 2^(Ew+E) at most).  That is relative
+// to the tile's largest value, not to what a node reads, so each node's sum |w||v|
 // is formed beside it in float32, and a node where it is below 2^(E-11) sum|w|
 // for some row leaves the digits: a result's error is at most about 2^-52
-// sum |w||v|, where a chain of FP64 fused multiply-adds has that for every
-// partial sum (measured: see kFloor).  The nodes
-// that leave, and all of a tile that holds an infinity or NaN, whose exponent is
-// extreme, or whose products do not come in time, are formed in FP64 by the
-// tile's CTA as the general kernels do.
+// sum |w||v|, where a chain of FP64 fused multiply-adds can round every partial
+// sum by 2^-53 of it (measured: see kFloor).  The nodes that leave, and all of a
+// tile that holds an infinity or NaN, whose exponent is extreme, or whose
+// products do not come in time, are formed in FP64 by the tile's CTA as the
+// general kernels do.
 //
 // Which nodes: `cls` of the plan.  Fictitious nodes (alpha-scaled rows) read
 // values far below their tile's largest in nearly every field (sum |w||v| from
