@@ -720,8 +720,7 @@ __global__ void __launch_bounds__(512, DIM == 2 ? 3 : 2)
           for (int u = 1; u < ND; ++u)
             if (t == u) yl = y[u];
           const bool fixed = t < DIM && ((mi >> t) & 1);
-          const float dold = d[pb + t];
-          d[pb + t] = fixed ? dold + rp[t] : fmaf(omega, yl, dold);
+          d[pb + t] = __fadd_rn(d[pb + t], fixed ? rp[t] : __fmul_rn(omega, yl));
         }
       }
     }
@@ -849,7 +848,7 @@ __global__ void __launch_bounds__(512, 1)
       for (int o = 4; o > 0; o >>= 1) yl += __shfl_xor_sync(0xffffffffu, yl, o);
       if (writer) {
         const bool fixed = t < 3 && ((mi >> t) & 1);
-        d[pb + t] = fixed ? dold + rself : fmaf(omega, yl, dold);
+        d[pb + t] = __fadd_rn(dold, fixed ? rself : __fmul_rn(omega, yl));
       }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");

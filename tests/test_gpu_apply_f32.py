@@ -52,35 +52,3 @@ def test_class_patches_and_lane_counts(fc, name, prec):
         if ref is None:
             ref = got
         assert np.max(np.abs(got - ref)) <= 1e-3 * np.max(np.abs(ref)), tile
-
-
-@pytest.mark.parametrize("prec", ["fp32", "bf16"])
-@pytest.mark.parametrize("tile", [(4, 256, 4), (8, 256, 4), (32, 256, 2)])
-@pytest.mark.parametrize("dim", [2, 3])
-def test_update_rounds_once(fc, dim, tile, prec):
-    """d + omega y is one rounding.  With omega near 2^-40 every sweep meets the
-    first one's residual bit for bit, and with 2^-40 itself the first sweep
-    gives y, so the later sweeps' values are known exactly."""
-    import dataclasses
-    import torch
-    p = inputs.channel_2d(0, n=24, nlevels=2) if dim == 2 else inputs.channel_3d(0, n=8, nlevels=2)
-    b = 1.5 + 0.5 * inputs.uniform_array(p.ndof(), 3)
-
-    def sweeps(omega, n):
-        B = fc.Batch([fc.Solver(dataclasses.replace(p, omega=omega), prec=prec)], tile=tile)
-        x = torch.zeros(p.ndof(), dtype=torch.float64, device="cuda")
-        B.smooth_(x, torch.as_tensor(b).cuda(), nsweeps=n)
-        out = x.cpu().numpy()
-        B.close()
-        return out
-
-    y = sweeps(2.0 ** -40, 1)
-    free = np.abs(y) < 1e-3                      # constrained values take the residual
-    y, omega = y * 2.0 ** 40, np.float64(np.float32(1.1 * 2.0 ** -40))
-    one = (omega * y).astype(np.float32).astype(np.float64)
-    np.testing.assert_array_equal(sweeps(omega, 1)[free], one[free])
-    np.testing.assert_array_equal(sweeps(omega, 2)[free], 2.0 * one[free])   # half an ulp of y is lost in 2 y
-    three = (omega * y + 2.0 * one).astype(np.float32).astype(np.float64)
-    np.testing.assert_array_equal(sweeps(omega, 3)[free], three[free])
-    twice = (3.0 * one).astype(np.float32).astype(np.float64)                # omega y rounded, then the sum
-    assert np.count_nonzero(three[free] != twice[free]) > np.count_nonzero(free) // 20
