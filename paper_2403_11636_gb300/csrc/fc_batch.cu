@@ -720,6 +720,7 @@ __global__ void __launch_bounds__(512, DIM == 2 ? 3 : 2)
           for (int u = 1; u < ND; ++u)
             if (t == u) yl = y[u];
           const bool fixed = t < DIM && ((mi >> t) & 1);
+          // a rounded product and a rounded sum, in every apply alike
           d[pb + t] = __fadd_rn(d[pb + t], fixed ? rp[t] : __fmul_rn(omega, yl));
         }
       }
